@@ -81,7 +81,8 @@ struct fcs_params {
   int device = -1;
   ParamDev d{};
   float* w = nullptr;           // device shape weights (the tables' source)
-  int32_t* bad = nullptr;       // per-entry flags of the table build
+  uint8_t* built = nullptr;     // per entry: its tables belong to the present weights
+  int32_t* list = nullptr;      // [n_entries + 1] entries to build and, last, their number
   uint32_t* check = nullptr;    // validation word of fcs_update_params
   std::vector<void*> allocs;
   ~fcs_params() {
@@ -588,7 +589,7 @@ int enqueue_call(const CallArgs& a, bool sync_size, const HitCfg& hc, int key_ta
 HitCfg hit_cfg(const fcs_config& c) {
   HitCfg h;
   h.block = c.block ? c.block : 128;  // the shape fcs_autotune picks on GB300 for pile-up batches
-  h.hpt = c.hits_per_thread ? c.hits_per_thread : 8;
+  h.hpt = c.hits_per_thread;  // 0: the kernel sizes its tickets from the hits
   h.det = c.mode == FCS_MODE_DETERMINISTIC;
   return h;
 }
@@ -827,6 +828,7 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
   int64_t cells = 0;
   std::vector<RegionF> rf(n_regions);
   std::vector<float> split32(n_regions);
+  std::vector<float4> grids(n_layers);
   std::vector<double> eta_lo(n_regions), deta(n_regions), phi_lo(n_regions), dphi(n_regions), split(n_regions);
   std::vector<int32_t> ne(n_regions), np(n_regions), co(n_regions);
   for (int l = 0; l < n_layers; ++l) {
@@ -862,18 +864,68 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
       }
       RegionF& f = rf[r];
       f = RegionF{};
-      f.ek = (float)(-g.eta_lo / g.deta);
+      const double ek = -g.eta_lo / g.deta, pk = -g.phi_lo / g.dphi;
+      f.ek = (float)ek;
       f.inv_deta = (float)(1.0 / g.deta);
-      f.pk = (float)(-g.phi_lo / g.dphi);
+      f.pk = (float)pk;
+      f.pkh = (float)(pk - 0.5);
       f.inv_dphi = (float)(1.0 / g.dphi);
       split32[r] = (float)split[r];
       f.n_eta_hf = (float)g.n_eta - 0.5f;
-      // bounds of the FP32 index beyond the position's error (fcs_hits.cuh: fast_cell), rounded up
-      f.ce = (float)(std::fabs((double)f.ek) * 0x1p-23 + 0x1p-22) * 1.0001f;
-      f.cp = (float)(std::fabs((double)f.pk) * 0x1p-23 + 0x1p-22) * 1.0001f;
+      // overlapping neighbours (up to 1e-9): a boundary deeper than 2^-22 of a
+      // cell inside a grid leaves both regions to the search
+      if (r > lrb[l]) {
+        const double in_this = (split[r] - g.eta_lo) / g.deta;
+        const fcs_region& p = regions[r - 1];
+        const double in_prev = (eta_lo[r - 1] + (double)p.n_eta * p.deta - split[r]) / p.deta;
+        if (in_this > 0x1p-22) f.fast_off = 1.0f;
+        if (in_prev > 0x1p-22) rf[r - 1].fast_off = 1.0f;
+      }
+      // bounds of the FP32 index beyond the position's error (fcs_hits.cuh: generic_cell), rounded up
+      f.ce = (float)(std::fabs(ek) * 0x1p-23 + 0x1p-22) * 1.0001f;
+      f.cp = (float)(std::fabs(pk) * 0x1p-23 + 0x1p-22) * 1.0001f;
       f.n_phi = g.n_phi;
       f.cell_off = g.cell_offset;
     }
+    // Neighbouring regions whose grids continue one another (the same phi grid
+    // and eta step, edges that meet within 2^-23 of a cell) are one grid for
+    // the hit kernel's staged map: fewer hits leave it, and a layer's mirrored
+    // halves are one.
+    const float inf = std::numeric_limits<float>::infinity();
+    float bound[3] = {inf, inf, inf};
+    uint32_t member = 0;
+    int n_grids = 0;
+    for (int a = lrb[l], b; a < lrb[l + 1]; a = b) {
+      if (n_grids < 4) {
+        if (n_grids > 0) bound[n_grids - 1] = split32[a];
+        member |= (uint32_t)a << (8 * n_grids);
+      }
+      ++n_grids;
+      const fcs_region& ga = regions[a];
+      int64_t n = ga.n_eta;
+      float off = rf[a].fast_off;
+      for (b = a + 1; b < lrb[l + 1]; ++b) {
+        const fcs_region& gb = regions[b];
+        if (gb.n_phi != ga.n_phi || gb.phi_lo != ga.phi_lo || gb.dphi != ga.dphi || gb.deta != ga.deta ||
+            std::fabs(gb.eta_lo - (ga.eta_lo + (double)n * ga.deta)) > 0x1p-23 * ga.deta || n + gb.n_eta > (1 << 22))
+          break;
+        n += gb.n_eta;
+        off = std::max(off, rf[b].fast_off);
+      }
+      for (int r = a; r < b; ++r) {
+        RegionF& f = rf[r];
+        f.ekh = (float)(-ga.eta_lo / ga.deta - 0.5);
+        f.n_eta = (float)n;
+        f.lo = a == lrb[l] ? 0.0f : -0.5f;
+        f.hi = f.n_eta - (b == lrb[l + 1] ? 1.0f : 0.5f);
+        f.fast_off = off;
+        f.fast_cell = ga.cell_offset;
+      }
+    }
+    float member_bits;
+    std::memcpy(&member_bits, &member, sizeof(float));
+    grids[l] = n_grids <= 4 ? make_float4(bound[0], bound[1], bound[2], member_bits)
+                            : make_float4(std::numeric_limits<float>::quiet_NaN(), inf, inf, 0.0f);
   }
   fcs_geo* geo = new fcs_geo();
   int rc = FCS_OK;
@@ -885,6 +937,7 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
   RegionF* d_rf;
   double *d_el, *d_de, *d_pl, *d_dp, *d_sp, *d_rz;
   float *d_rinv32, *d_sp32;
+  float4* d_grids;
   int32_t *d_ne, *d_np, *d_co, *d_lrb, *d_bar;
   if ((rc = dev_alloc(&d_rf, n_regions, &geo->allocs)) || (rc = dev_alloc(&d_el, n_regions, &geo->allocs)) ||
       (rc = dev_alloc(&d_de, n_regions, &geo->allocs)) || (rc = dev_alloc(&d_pl, n_regions, &geo->allocs)) ||
@@ -892,7 +945,8 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
       (rc = dev_alloc(&d_ne, n_regions, &geo->allocs)) || (rc = dev_alloc(&d_np, n_regions, &geo->allocs)) ||
       (rc = dev_alloc(&d_co, n_regions, &geo->allocs)) || (rc = dev_alloc(&d_lrb, n_layers + 1, &geo->allocs)) ||
       (rc = dev_alloc(&d_rz, n_layers, &geo->allocs)) || (rc = dev_alloc(&d_bar, n_layers, &geo->allocs)) ||
-      (rc = dev_alloc(&d_rinv32, n_layers, &geo->allocs)) || (rc = dev_alloc(&d_sp32, n_regions, &geo->allocs)))
+      (rc = dev_alloc(&d_rinv32, n_layers, &geo->allocs)) || (rc = dev_alloc(&d_sp32, n_regions, &geo->allocs)) ||
+      (rc = dev_alloc(&d_grids, n_layers, &geo->allocs)))
     return fail(rc);
   std::vector<double> rz(n_layers);
   std::vector<float> rinv32(n_layers);
@@ -912,7 +966,8 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
                 {d_ne, ne.data(), n_regions * sizeof(int32_t)},   {d_np, np.data(), n_regions * sizeof(int32_t)},
                 {d_co, co.data(), n_regions * sizeof(int32_t)},   {d_lrb, lrb, (n_layers + 1) * sizeof(int32_t)},
                 {d_rz, rz.data(), n_layers * sizeof(double)},     {d_bar, bar.data(), n_layers * sizeof(int32_t)},
-                {d_rinv32, rinv32.data(), n_layers * sizeof(float)},  {d_sp32, split32.data(), n_regions * sizeof(float)}};
+                {d_rinv32, rinv32.data(), n_layers * sizeof(float)},  {d_sp32, split32.data(), n_regions * sizeof(float)},
+                {d_grids, grids.data(), n_layers * sizeof(float4)}};
   for (const auto& c : copies) {
     cudaError_t e = cudaMemcpyAsync(c.d, c.h, c.n, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return fail(set_err(FCS_E_CUDA, "geometry copy: %s", cudaGetErrorString(e)));
@@ -931,6 +986,7 @@ int fcs_load_geometry(fcs_geo** out, const fcs_region* regions, int32_t n_region
   d.dphi = d_dp;
   d.split = d_sp;
   d.split32 = d_sp32;
+  d.grids = d_grids;
   d.n_eta = d_ne;
   d.n_phi = d_np;
   d.cell_off = d_co;
@@ -998,8 +1054,7 @@ int fcs_load_params(fcs_params** out, const fcs_geo* geo, const float* frac, con
   float *d_frac, *d_mhe, *d_re, *d_ae, *d_lf, *d_w = nullptr;
   double* d_lf64 = nullptr;
   uint32_t* d_thr;
-  uint2* d_guide;
-  int32_t* d_bad = nullptr;
+  uint32_t* d_guide;
   if ((rc = dev_alloc(&d_frac, n_entries, &prm->allocs)) || (rc = dev_alloc(&d_mhe, n_entries, &prm->allocs)) ||
       (rc = dev_alloc(&d_re, NR + 1, &prm->allocs)) || (rc = dev_alloc(&d_ae, NA + 1, &prm->allocs)) ||
       (rc = dev_alloc(&d_thr, n_entries * kNBins, &prm->allocs)) ||
@@ -1015,7 +1070,8 @@ int fcs_load_params(fcs_params** out, const fcs_geo* geo, const float* frac, con
     lf64[k] = std::lgamma((double)k + 1.0);
     lf[k] = (float)lf64[k];
   }
-  if ((rc = dev_alloc(&d_w, n_entries * kNBins, &prm->allocs)) || (rc = dev_alloc(&d_bad, n_entries, &prm->allocs)) ||
+  if ((rc = dev_alloc(&d_w, n_entries * kNBins, &prm->allocs)) || (rc = dev_alloc(&prm->built, n_entries, &prm->allocs)) ||
+      (rc = dev_alloc(&prm->list, n_entries + 1, &prm->allocs)) ||
       (rc = dev_alloc(&prm->check, 1, &prm->allocs)))
     return fail(rc);
   cudaError_t e = cudaSuccess;
@@ -1027,12 +1083,12 @@ int fcs_load_params(fcs_params** out, const fcs_geo* geo, const float* frac, con
       (e = cudaMemcpyAsync(d_lf64, lf64.data(), kLfactEntries * sizeof(double), cudaMemcpyHostToDevice, s)) !=
           cudaSuccess ||
       (e = cudaMemcpyAsync(d_w, shape_w, n_entries * kNBins * sizeof(float), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = launch_build_tables(d_w, (int)n_entries, d_thr, d_guide, d_bad, s)) != cudaSuccess ||
+      (e = launch_build_tables(d_frac, d_w, (int)n_entries, 1, prm->built, prm->list, prm->list + n_entries, d_thr,
+                               d_guide, s)) != cudaSuccess ||
       (e = cudaStreamSynchronize(s)) != cudaSuccess) {
     return fail(set_err(FCS_E_CUDA, "parametrisation upload: %s", cudaGetErrorString(e)));
   }
   prm->w = d_w;
-  prm->bad = d_bad;
   ParamDev& d = prm->d;
   d.NT = NT;
   d.NE = NE;
@@ -1078,10 +1134,13 @@ int fcs_update_params(fcs_params* prm, const float* frac, const float* mean_hit_
   if (bad & 8u) return set_err(FCS_E_ARG, "shape_w of an entry with frac > 0 sums to 0");
   if (frac) FCS_CUDA(cudaMemcpyAsync((void*)d.frac, frac, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
   if (mean_hit_E) FCS_CUDA(cudaMemcpyAsync((void*)d.mhe, mean_hit_E, n * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  if (shape_w) {
+  if (shape_w)
     FCS_CUDA(cudaMemcpyAsync(prm->w, shape_w, n * kNBins * sizeof(float), cudaMemcpyDeviceToDevice, s));
-    FCS_CUDA(launch_build_tables(prm->w, (int)n, (uint32_t*)d.thr, (uint2*)d.guide, prm->bad, s));
-  }
+  // new weights: the tables of every entry with a fraction; new fractions
+  // alone: those of the entries that had none when the weights came
+  if (shape_w || frac)
+    FCS_CUDA(launch_build_tables(d.frac, prm->w, (int)n, shape_w ? 1 : 0, prm->built, prm->list, prm->list + n,
+                                 (uint32_t*)d.thr, (uint32_t*)d.guide, s));
   return ok();
 }
 

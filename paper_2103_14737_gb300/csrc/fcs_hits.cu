@@ -34,6 +34,4 @@ cudaError_t launch_recheck(const GeoDev& g, const ParamDev& p, WsDev w, int32_t 
   return det ? launch_recheck_t<kModeDet>(kp, L) : launch_recheck_t<kModeAtomic>(kp, L);
 }
 
-int hits_max_smem_tasks() { return kSmemTasks; }
-
 }  // namespace fcs

@@ -4,30 +4,30 @@
 // One thread per hit as in the paper's sim_a kernel (Sec. 4), but persistent:
 // CTAs take tiles of BLOCK * HPT consecutive hits from an atomic work queue
 // over the whole batch (the grouped simulation of Sec. 4 at batch scale); a
-// tile's task records are staged in shared memory and each hit finds its task
-// through a block max-scan of task start positions.  Per hit:
+// tile's tasks are staged in shared memory, each with its hits' map to scaled
+// cell indices folded into one multiply-add per coordinate, and each hit finds
+// its task by counting the task starts at or before it.  Per hit:
 //   Philox4x32-10 block (hit, layer, particle, event)        -> 4 words
 //   word 0: shape bin by guide table + binary search          (integer, exact)
 //   words 1, 2: uniform position in the (r, alpha) bin        (FP32)
-//   (r, alpha) -> (eta, phi) linear map around the task centre (FP32, __sincosf)
-//   region search + grid index                                 (FP32)
-// The FP32 result is certified against a rigorous error bound; a hit whose
-// eta or phi lies within the bound of a cell or region edge is queued and
-// decided by the FP64 recheck kernel, which repeats the oracle's FP64 steps
-// (the paper's two FP32 cell mismatches in 62M hits were removed with FP64,
-// Sec. 6).  Certified hits are deposited with warp-aggregated atomics (Sec. 4
-// chose atomicAdd) of the float count x Ehit into FP64 cells or, in
-// deterministic mode, emitted as (cell, task, count) records for the
-// sort-by-cell reduction.
+//   (r, alpha) -> scaled (eta, phi) cell indices of the task's home region
+//     (FP32, __sincosf)
+// The FP32 result is certified against a rigorous error bound.  A hit that
+// leaves the home region or lies within the bound of a cell edge (about one in
+// 200) takes the search over the layer's regions, certified likewise; what
+// stays uncertain (one in 5000) is queued and decided by the FP64 recheck
+// kernel, which repeats the oracle's FP64 steps (the paper's two FP32 cell
+// mismatches in 62M hits were removed with FP64, Sec. 6).  Certified hits are
+// deposited with warp-aggregated atomics (Sec. 4 chose atomicAdd) of the float
+// count x Ehit into FP64 cells or, in deterministic mode, emitted as (cell,
+// task, count) records for the sort-by-cell reduction.
 #pragma once
-
-#include <type_traits>
 
 #include "fcs_internal.cuh"
 
 namespace fcs {
 
-constexpr int kSmemTasks = 128;  // staged tasks per tile (more: the hit loop reads the records)
+constexpr int kMaxTicket = 1024;  // hits a warp takes from the work queue at a time, at most
 
 struct HitKParams {
   GeoDev g;
@@ -37,7 +37,7 @@ struct HitKParams {
   uint32_t k0, k1;
   uint32_t first_event_lo;
   int32_t key_task_bits;
-  int32_t key32;  // 32-bit (cell, task-in-tile) match keys (n_cells < 2^19)
+  int32_t key32;  // 32-bit (cell, task in pass) match keys (n_cells < 2^27)
   int32_t* dbg_hit_cell;
   int16_t* dbg_hit_bin;
   int64_t dbg_hit_cap;
@@ -45,8 +45,9 @@ struct HitKParams {
   const float* grad_in;  // dL/dE_cell of the range's events, row stride n_cells
   double* grad_acc;      // [n_entries][128] sum of E_hit dL/dE_cell per (entry, shape bin)
   uint8_t* grad_touched; // [n_entries] set where grad_acc has contributions
-  // one launch per task (static_tiles != 0): CTA b takes tile b of the hits
-  // [h_lo, h_hi), all of task t_last
+  int32_t ticket;        // hits per queue ticket, a multiple of kGranule up to kMaxTicket; 0: from the call's hits
+  // one launch per task (static_tiles != 0): warp b of the grid takes tile b
+  // of the hits [h_lo, h_hi), all of task t_last
   int64_t h_lo, h_hi;
   int32_t t_last;
   int32_t static_tiles;
@@ -54,31 +55,51 @@ struct HitKParams {
 };
 
 // ---- shape bin: inverse CDF by guide table and binary search --------------
-// Binary search for the first k in [lo, hi) with x0 < T[k], else hi.
-static __device__ __noinline__ int bin_search(const uint32_t* T, int lo, int hi, uint32_t x0) {
+// The bin of word x0 for an entry whose bins below lo lie below x0: the first
+// k >= lo with x0 < T[k].  T is 2^32 - 1 from the last bin K
+// of non-zero weight on, so K is found for every word but 2^32 - 1, which is
+// below no threshold and belongs to K.
+static __device__ __noinline__ int bin_search(const ParamDev& p, uint32_t gbase, int lo, uint32_t x0) {
+  if (x0 == 0xFFFFFFFFu) {
+    int k = kNBins - 1;
+    while (k > 0 && !(__ldg(p.shape_w + gbase + k) > 0.0f)) --k;
+    return k;
+  }
+  // most searches end within four thresholds: they are loaded at once
+  int n = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) n += x0 >= __ldg(p.thr + gbase + min(lo + j, kNBins - 1)) ? 1 : 0;
+  lo += n;
+  if (n < 4) return lo;
+  int hi = kNBins - 1;
   while (lo < hi) {
     const int mid = (lo + hi) >> 1;
-    if (x0 < __ldg(T + mid)) hi = mid;
+    if (x0 < __ldg(p.thr + gbase + mid)) hi = mid;
     else lo = mid + 1;
   }
   return lo;
 }
 
-// The bin of word x0: the packed guide cell of x0's top 7 bits gives lo and
-// the first two thresholds of the cell as offsets (fcs_params.cu); two
-// comparisons decide unless the cell spans three or more bins and x0 lies
-// past the second threshold (a few percent of the words), which finishes with
-// a binary search over the thresholds.
-__device__ __forceinline__ int sample_bin(const ParamDev& p, int32_t entry, uint32_t x0) {
-  const uint2 gg = __ldg(p.guide + ((uint32_t)entry * kGuideCells + (x0 >> 25)));
-  const uint32_t xo = x0 & 0x1FFFFFFu;
-  const uint32_t t0 = gg.x & 0x1FFFFFFu;
-  const uint32_t t1 = __funnelshift_r(gg.x, gg.y, 25) & 0x1FFFFFFu;
-  const int lo = (int)((gg.y >> 18) & 0x7Fu);
-  const int bin = lo + (xo > t0 ? 1 : 0) + (xo > t1 ? 1 : 0);
-  const int span = (int)(gg.y >> 25);
-  if (span > 2 && xo > t1) return bin_search(p.thr + (uint32_t)entry * kNBins, lo + 2, lo + span, x0);
-  return bin;
+// The bin of word x0: the guide cell of x0's top 8 bits gives lo and the
+// cell's first threshold as an offset (fcs_params.cu); one comparison decides
+// unless the cell holds two or more thresholds and x0 lies past the first (two
+// words in a hundred), which finishes with a binary search over the
+// thresholds.  gbase: the entry x 128 (its first threshold; its first guide
+// cell is 2 gbase).
+struct GuideBin {
+  int bin;      // the bin, or the first bin of the search
+  bool search;
+};
+__device__ __forceinline__ uint32_t guide_word(const ParamDev& p, uint32_t gbase, uint32_t x0) {
+  return __ldg(p.guide + (2u * gbase + (x0 >> 24)));
+}
+__device__ __forceinline__ GuideBin bin_in_cell(uint32_t x0, uint32_t g) {
+  const bool past = (x0 << 8) > g;  // x0 past the threshold (the low byte of g does not reach the offset's bits)
+  return {(int)((g >> 1) & 0x7Fu) + (past ? 1 : 0), past && (g & 1u)};
+}
+__device__ __forceinline__ int sample_bin(const ParamDev& p, uint32_t gbase, uint32_t x0) {
+  const GuideBin b = bin_in_cell(x0, guide_word(p, gbase, x0));
+  return b.search ? bin_search(p, gbase, b.bin, x0) : b.bin;
 }
 
 // ---- FP64 path: the oracle's steps, each rounding once ----------------------
@@ -134,41 +155,17 @@ static __device__ __noinline__ int32_t cell_fp64(const GeoDev& g, const ParamDev
   return lookup64(g, layer, eta, phi);
 }
 
-// ---- shared tables of a CTA ---------------------------------------------------
-struct HitSmemTables {
-  RegionF reg[kMaxRegions];
-  float split[kMaxRegions];  // lower ownership boundary of each region (FP32)
-  int32_t lrb[kMaxLayers + 1];
-  float4 rb[kNR];  // r bin: lo, width, hi, hi 2^-17 (the bin's term of the error bound)
-  float2 ab[kNA];  // alpha bin: lo - pi, width
-};
-
-__device__ __forceinline__ void load_tables(HitSmemTables& t, const GeoDev& g, const ParamDev& p) {
-  for (int i = threadIdx.x; i < g.n_regions; i += blockDim.x) {
-    t.reg[i] = g.regf[i];
-    t.split[i] = g.split32[i];
-  }
-  for (int i = threadIdx.x; i <= g.n_layers; i += blockDim.x) t.lrb[i] = g.lrb[i];
-  if (threadIdx.x < kNR) {
-    const float lo = p.r_edges[threadIdx.x], hi = p.r_edges[threadIdx.x + 1];
-    t.rb[threadIdx.x] = make_float4(lo, hi - lo, hi, hi * 0x1p-17f);
-  }
-  if (threadIdx.x < kNA) {
-    const double lo = p.a_edges[threadIdx.x], hi = p.a_edges[threadIdx.x + 1];
-    t.ab[threadIdx.x] = make_float2((float)(lo - 3.141592653589793), (float)(hi - lo));
-  }
-}
-
-// ---- FP32 fast path --------------------------------------------------------
+// ---- search over the layer's regions (FP32, certified) -------------------------
+// For the hits that the staged map of the home region cannot certify.
 // Error bound of the FP32 eta (and likewise phi) against the FP64 value:
-//   cos/sin: |alpha32 - alpha| <= ~2^-21.4 (alpha - pi in [-pi, pi] from an
-//     FMA of FP32 table values) and __sincosf's documented absolute error on
-//     [-pi, pi] (2^-21.19 for cos, 2^-21.41 for sin): <= 2^-20.4 in all;
+//   cos/sin: |alpha32 - alpha| <= ~2^-21 (alpha - pi in [-pi, pi] from an
+//     FMA of FP32 values) and __sincosf's documented absolute error on
+//     [-pi, pi] (2^-21.19 for cos, 2^-21.41 for sin): <= 2^-20 in all;
 //   r32 <= r_hi * 2^-23 off; s32 (coshf, sinhf and tanhf within 2, 3 and 2
 //     ulp as documented, a correctly rounded 1/R or 1/cosh and up to two
 //     products: <= 8 ulp) <= 2^-20 relative; the two products 2 * 2^-24
 //     relative:
-//   => |deta32 - deta| <= r_hi |s_eta| 2^-19; bound used: r_hi |s| 2^-17;
+//   => |deta32 - deta| <= r_hi |s_eta| 2^-18.8; bound used: r_hi |s| 2^-17;
 //   the final add rounds by |eta| 2^-24; bound used: |eta| 2^-21.
 // Scaled index te = fl(eta32 inv + ek) with inv = fl(1/deta), ek =
 // fl(-eta_lo/deta): |te - te*| <= be inv + (|eta| inv) 2^-24 + |ek| 2^-24 +
@@ -178,104 +175,31 @@ __device__ __forceinline__ void load_tables(HitSmemTables& t, const GeoDev& g, c
 // phi).
 // A decision is certified when the FP32 value is farther than the bound
 // (plus the FP32 rounding of the boundary) from the boundary it is compared
-// with.
-struct FastHit {
-  int32_t cell;
-  bool sure;
-};
-
-// The regions [a, b) of a task's layer that its hits can reach: every hit
-// lies within r_max |s_eta| of eta_c in eta (r_max = the outer edge of the
-// shape histogram), widened by 2^-8 relative and 2^-16 (1 + |eta_c|) for the
-// FP32 scale factor and for the rounding of the FP32 and FP64 hit positions.
-// Split q is left out of the search when the FP64 split lies below (above)
-// every hit, judged from its FP32 copy with a 2^-22 relative margin, so the
-// search over [a, b) decides exactly as the search over the whole layer and
-// needs no certification at the splits it skips.
-__device__ __forceinline__ uint32_t task_lay(const HitSmemTables& tb, int layer, float eta_c, float s_eta) {
-  const int rb = tb.lrb[layer], re = tb.lrb[layer + 1];
-  const float D = fmaf(tb.rb[kNR - 1].z * fabsf(s_eta), 1.00390625f, fmaf(fabsf(eta_c), 0x1p-16f, 0x1p-16f));
-  const float L = eta_c - D, U = eta_c + D;
-  int a = rb, b = re;
-  for (int q = rb + 1; q < re; ++q) {
-    const float sp = tb.split[q];
-    if (fmaf(fabsf(sp), 0x1p-22f, sp) <= L) a = q;
-    if (b == re && fmaf(-fabsf(sp), 0x1p-22f, sp) > U) b = q;
-  }
-  return (uint32_t)layer | ((uint32_t)a << 8) | ((uint32_t)b << 20);
-}
-
-// A task as the hit loop uses it, staged in shared memory per tile (48 B):
-// 32-bit offsets and the Philox counter words are formed once per task.
-struct TileTask {
-  int32_t rel;      // first hit of the task - first hit of the tile (<= 0 for the tile's first task)
-  int32_t entry;    // parametrisation entry (with layer)
-  float Ehit, eta_c, phi_c, s_eta, s_phi;
-  uint32_t ctr_y;   // layer | purpose << 16
-  uint32_t ctr_z;   // particle in event
-  uint32_t ctr_w;   // event number of the random stream
-  uint32_t row_off; // row * acc_stride (atomic, deterministic) or row * n_cells (gradient)
-  uint32_t lay;     // layer | first region << 8 | end region << 20 (the reachable regions)
-};
-static_assert(sizeof(TileTask) == 48, "TileTask layout");
-
-// The tile's view of task t: hit offset relative to the tile start h0, the
-// float hit energy fl32(El / n), the Philox counter words and the accumulation
-// row.
-__device__ __forceinline__ TileTask make_tile_task(const HitSmemTables& tb, const WsDev& w, int64_t t, int64_t h0,
-                                                   uint32_t first_event_lo, int32_t ev_lo, uint32_t row_stride) {
-  const TaskRec r = w.tasks[t];
-  const int32_t layer = r.layer(), event = r.event();
-  TileTask q;
-  q.rel = (int32_t)(w.th[t] - h0);
-  q.entry = r.entry;
-  q.Ehit = __fdiv_rn(r.El, (float)w.tn[t]);
-  q.eta_c = r.eta_c;
-  q.phi_c = r.phi_c;
-  q.s_eta = r.s_eta;
-  q.s_phi = r.s_phi;
-  q.ctr_y = (uint32_t)layer | (kPurposeHit << 16);
-  q.ctr_z = (uint32_t)r.particle;
-  q.ctr_w = first_event_lo + (uint32_t)event;
-  q.row_off = (uint32_t)(event - ev_lo) * row_stride;
-  q.lay = task_lay(tb, layer, r.eta_c, r.s_eta);
-  return q;
-}
-
-template <typename TT>
-__device__ __forceinline__ FastHit fast_cell(const HitSmemTables& tb, const TT& T, uint4 x, int bin) {
+// with.  Returns the cell, or -1 when a decision is not certified.
+__device__ __forceinline__ int32_t generic_cell(const GeoDev& g, const ParamDev& p, const TaskRec& T, uint4 x,
+                                                int bin) {
   const int ir = bin >> 3, ia = bin & 7;
-  const float ur = u24f(x.y), ua = u24f(x.z);
-  const float4 rbin = tb.rb[ir];
-  const float2 abin = tb.ab[ia];
-  const float r = fmaf(ur, rbin.y, rbin.x);
-  const float ap = fmaf(ua, abin.y, abin.x);  // alpha - pi
+  const float r_lo = __ldg(p.r_edges + ir), r_hi = __ldg(p.r_edges + ir + 1);
+  const float a_lo = __ldg(p.a_edges + ia), a_hi = __ldg(p.a_edges + ia + 1);
+  const float r = fmaf(u24f(x.y), r_hi - r_lo, r_lo);
+  // alpha - pi (pi in two floats; within one more rounding of the FP64 difference)
+  const float ap = fmaf(u24f(x.z), a_hi - a_lo, (a_lo - 3.14159274f) + 8.74227766e-8f);
   float sn, cs;
   __sincosf(ap, &sn, &cs);
-  const float de = (r * -cs) * T.s_eta;
-  const float dp = (r * -sn) * T.s_phi;
-  const float eta = T.eta_c + de;
-  const float phi = T.phi_c + dp;
+  const float eta = T.eta_c + (r * -cs) * T.s_eta;
+  const float phi = T.phi_c + (r * -sn) * T.s_phi;
   // the bounds r_hi |s| 2^-17 + |x| 2^-21 of the FP32 eta and phi
-  const float be = fmaf(rbin.w, fabsf(T.s_eta), fabsf(eta) * 0x1p-21f);
-  const float bp = fmaf(rbin.w, fabsf(T.s_phi), fabsf(phi) * 0x1p-21f);
+  const float be = fmaf(r_hi * 0x1p-17f, fabsf(T.s_eta), fabsf(eta) * 0x1p-21f);
+  const float bp = fmaf(r_hi * 0x1p-17f, fabsf(T.s_phi), fabsf(phi) * 0x1p-21f);
   bool sure = fabsf(eta) < 1.0e30f;  // false for NaN or huge eta (a NaN phi fails its own test below)
-  // region: the last of the task's reachable regions [rb, re) whose split lies
-  // at or below eta.  Most tasks reach one region or two (one split, tested
-  // without a branch); a loop takes the further splits.
-  const int rb = (T.lay >> 8) & 0xFFF, re = T.lay >> 20;
-  const bool two = re > rb + 1;
-  const float sp1 = tb.split[min(rb + 1, kMaxRegions - 1)];  // read by every lane, used where two
-  int rr = (two && eta >= sp1) ? rb + 1 : rb;
-  sure &= !two || fabsf(eta - sp1) > fmaf(fabsf(sp1), 0x1p-23f, be);
-  if (re > rb + 2) {
-    for (int q = rb + 2; q < re; ++q) {
-      const float sp = tb.split[q];
-      if (eta >= sp) rr = q;
-      sure &= fabsf(eta - sp) > fmaf(fabsf(sp), 0x1p-23f, be);
-    }
+  const int layer = T.layer(), rb = __ldg(g.lrb + layer), re = __ldg(g.lrb + layer + 1);
+  int rr = rb;
+  for (int q = rb + 1; q < re; ++q) {
+    const float sp = __ldg(g.split32 + q);
+    if (eta >= sp) rr = q;
+    sure &= fabsf(eta - sp) > fmaf(fabsf(sp), 0x1p-23f, be);
   }
-  const RegionF R = tb.reg[rr];
+  const RegionF R = g.regf[rr];
   // eta index, clamped to [1/2, n_eta - 1/2]: outside it the cell is the first
   // or the last whichever side of the region's edge the hit lies, and at the
   // clamp the distance to the nearest integer is 1/2, so only interior cell
@@ -287,16 +211,150 @@ __device__ __forceinline__ FastHit fast_cell(const HitSmemTables& tb, const TT& 
   const float tp = fmaf(phi, R.inv_dphi, R.pk);
   const float kp = rintf(tp);
   sure &= fabsf(tp - kp) > fmaf(fabsf(tp), 0x1p-21f, fmaf(bp, R.inv_dphi, R.cp));
-  int ip = (int)floorf(tp);
+  int ip = (int)floorf(tp) % R.n_phi;
   if (ip < 0) ip += R.n_phi;
-  else if (ip >= R.n_phi) ip -= R.n_phi;
-  if ((unsigned)ip >= (unsigned)R.n_phi) {  // more than one turn in phi: rare
-    ip %= R.n_phi;
-    if (ip < 0) ip += R.n_phi;
+  return sure ? R.cell_off + ie * R.n_phi + ip : -1;
+}
+
+// ---- staged tasks and the home region's map -----------------------------------
+// The r and alpha bins as one multiply-add of f = 1 + u', f in [1, 2) built
+// from the top 23 bits of a random word (u' = u without its last bit).
+struct HitSmemTables {
+  float2 rb[kNR];  // r = f rb.y + rb.x: lo - width, width
+  float2 ab[kNA];  // alpha - pi = f ab.y + ab.x
+};
+
+__device__ __forceinline__ void load_tables(HitSmemTables& t, const ParamDev& p) {
+  if (threadIdx.x < kNR) {
+    const float lo = p.r_edges[threadIdx.x], hi = p.r_edges[threadIdx.x + 1];
+    t.rb[threadIdx.x] = make_float2(lo - (hi - lo), hi - lo);
   }
+  if (threadIdx.x < kNA) {
+    const double lo = p.a_edges[threadIdx.x], hi = p.a_edges[threadIdx.x + 1];
+    const float w = (float)(hi - lo);
+    t.ab[threadIdx.x] = make_float2((float)(lo - 3.141592653589793 - (double)w), w);
+  }
+}
+
+// A task as the hit loop uses it (80 B).  With inv = 1 / deta, ekh = -eta_lo /
+// deta - 1/2 of the home region (and likewise phi), a hit's scaled index minus
+// 1/2 is
+//   te = (r cos(alpha - pi)) ea + eb,  ea = -s_eta inv,  eb = eta_c inv + ekh,
+// one product and one multiply-add, and rint(te) is its cell index; pb is
+// reduced by whole turns.  Bound of te's error, r eB + be + 1/2, with R the
+// outer edge of the shape histogram:
+//   r: u' is off by 2^-24; with the roundings of width, lo - width and the
+//     FMA <= 5 2^-24 R;
+//   alpha - pi: width w rounded (w - pi - lo formed with the rounded one),
+//     u', the constant and the FMA's rounding: <= 2^-19.9 for any bin (2^-21.5
+//     for the usual 8 bins); __sincosf 2^-21.19 absolute: <= 2^-19.4;
+//   s32: <= 2^-20 relative (generic_cell); inv and the products 3 2^-24:
+//   => r |ea| 2^-18.6 + R |ea| 5 2^-24; used: r |ea| 2^-17 + R |ea| 2^-21;
+//   eb: (|eta_c| inv + |ekh| + |eb|) 2^-24 with |eta_c| inv <= |eb| + |ekh|,
+//     and the FMA's rounding |te| 2^-24 <= n_eta 2^-24 wherever it decides
+//     (beyond, te is clamped): used (|eb| + |ekh| + n_eta) 2^-23;
+//   pb: likewise, and the reduction by whole turns rounds by n_phi 2^-23;
+//   2^-21 absorbs second-order terms, the roundings of the bound itself and
+//   neighbours' boundaries up to 2^-22 inside the grid (RegionF::fast_off).
+// be and bp carry -1/2, so that a hit is certain when |te - rint(te)| <
+// -(r eB + be), i.e. when its distance to the nearest cell edge exceeds the
+// bound; a NaN or infinity anywhere fails the test.
+struct __align__(16) TileTask {
+  int32_t rel;      // first hit of the task - first hit of the pass (<= 0 for its first task)
+  uint32_t gbase;   // parametrisation entry (with layer) x 128
+  float Ehit;
+  // Philox rounds 1 and 2 with the task's counter words folded in: only one
+  // 32 x 32-bit product of each round depends on the hit
+  uint32_t c0, c1, c2, c3;
+  uint32_t base;    // accumulation row and region offset: + ie n_phi + ip, ie biased by kMagicBits
+  int32_t n_phi;
+  float ea, eb, pa, pb;
+  float be, bp, eB, pB;
+  float lo, hi;     // clamp of te (RegionF)
+  float pad;
+};
+static_assert(sizeof(TileTask) == 80, "TileTask layout");
+
+constexpr float kMagic = 12582912.0f;           // 1.5 2^23: adding it rounds to the nearest integer,
+constexpr uint32_t kMagicBits = 0x4B400000u;    // which the low bits then hold (|x| < 2^22)
+
+// The warp's view of task t: hit offset relative to the pass's first hit h0, the
+// float hit energy fl32(El / n), the Philox counter words, the map and the
+// accumulation row.
+__device__ __forceinline__ TileTask make_tile_task(const WsDev& w, const GeoDev& g, int64_t t, int64_t h0,
+                                                   uint32_t first_event_lo, int32_t ev_lo, uint32_t row_stride,
+                                                   float r_max, const PhiloxRoundKeys& rk) {
+  const TaskRec r = w.tasks[t];
+  const RegionF R = g.regf[r.region()];
+  const int32_t layer = r.layer(), event = r.event();
+  TileTask q;
+  q.rel = (int32_t)(w.th[t] - h0);
+  q.gbase = (uint32_t)r.entry() * kNBins;
+  q.Ehit = __fdiv_rn(r.El, (float)w.tn[t]);
+  {  // counter (hit, layer | purpose << 16, particle in event, event): round 1's second product, round 2's first
+    const uint32_t z = (uint32_t)r.particle;
+    const uint32_t x1 = __umulhi(kPhiloxM1, z) ^ ((uint32_t)layer | (kPurposeHit << 16)) ^ rk.k[0];
+    q.c0 = (first_event_lo + (uint32_t)event) ^ rk.k[1];
+    q.c1 = kPhiloxM1 * z ^ rk.k[2];
+    q.c2 = __umulhi(kPhiloxM0, x1) ^ rk.k[3];
+    q.c3 = kPhiloxM0 * x1;
+  }
+  q.n_phi = R.n_phi;
+  q.base = (uint32_t)(event - ev_lo) * row_stride + (uint32_t)R.fast_cell - kMagicBits * (uint32_t)R.n_phi;
+  q.ea = -r.s_eta * R.inv_deta;
+  q.eb = fmaf(r.eta_c, R.inv_deta, R.ekh);
+  q.pa = -r.s_phi * R.inv_dphi;
+  const float pb = fmaf(r.phi_c, R.inv_dphi, R.pkh);
+  const float nf = (float)R.n_phi;
+  q.pb = fmaf(-floorf(__fdividef(pb, nf)), nf, pb);
+  q.eB = fabsf(q.ea) * 0x1p-17f;
+  q.pB = fabsf(q.pa) * 0x1p-17f;
+  q.be = fmaf(fabsf(q.eb) + fabsf(R.ekh) + R.n_eta, 0x1p-23f, fmaf(r_max * fabsf(q.ea), 0x1p-21f, 0x1p-21f)) +
+         (R.fast_off - 0.5f);
+  q.bp = fmaf(fabsf(pb) + fabsf(R.pkh) + 2.0f * nf, 0x1p-23f, fmaf(r_max * fabsf(q.pa), 0x1p-21f, 0x1p-21f)) - 0.5f;
+  q.lo = R.lo;
+  q.hi = R.hi;
+  q.pad = 0.0f;
+  return q;
+}
+
+// The hit's Philox block from the task's folded words: rounds 1 and 2, then
+// the eight others.
+__device__ __forceinline__ uint4 hit_block(const TileTask& T, uint32_t hit, const PhiloxRoundKeys& rk) {
+  const uint32_t z1 = __umulhi(kPhiloxM0, hit) ^ T.c0, w1 = kPhiloxM0 * hit;
+  uint4 c = make_uint4(__umulhi(kPhiloxM1, z1) ^ T.c1, kPhiloxM1 * z1, w1 ^ T.c2, T.c3);
+#pragma unroll
+  for (int i = 2; i < 10; ++i) c = philox_round(c, rk.k[2 * i], rk.k[2 * i + 1]);
+  return c;
+}
+
+struct FastHit {
+  uint32_t cell;  // accumulation row offset + cell
+  bool sure;
+};
+
+__device__ __forceinline__ FastHit fast_cell(const HitSmemTables& tb, const TileTask& T, uint32_t x1, uint32_t x2,
+                                              int bin) {
+  const float2 rbin = tb.rb[bin >> 3], abin = tb.ab[bin & 7];
+  // the top 23 bits of a word below the exponent of 1.0f
+  const float r = fmaf(__uint_as_float(__funnelshift_r(x1, 0x7Fu, 9)), rbin.y, rbin.x);
+  const float ap = fmaf(__uint_as_float(__funnelshift_r(x2, 0x7Fu, 9)), abin.y, abin.x);  // alpha - pi
+  float sn, cs;
+  __sincosf(ap, &sn, &cs);
+  const float te = fminf(fmaxf(fmaf(r * cs, T.ea, T.eb), T.lo), T.hi);
+  const float tp = fmaf(r * sn, T.pa, T.pb);
+  const float ke = te + kMagic, kp = tp + kMagic;
   FastHit f;
-  f.cell = R.cell_off + ie * R.n_phi + ip;
-  f.sure = sure;
+  f.sure = fabsf(te - (ke - kMagic)) < -fmaf(r, T.eB, T.be) && fabsf(tp - (kp - kMagic)) < -fmaf(r, T.pB, T.bp);
+  // the phi index wrapped into [0, n_phi): as unsigned numbers, the smaller of
+  // ip and ip + n is ip + n exactly for ip < 0, that of ip and ip - n is ip - n
+  // exactly for ip >= n (one turn either way; beyond, the search takes the hit)
+  const uint32_t n = (uint32_t)T.n_phi;
+  uint32_t ip = __float_as_uint(kp) - kMagicBits;
+  ip = min(ip, ip + n);
+  ip = min(ip, ip - n);
+  f.sure = f.sure && ip < n;
+  f.cell = T.base + __float_as_uint(ke) * n + ip;
   return f;
 }
 
@@ -400,197 +458,281 @@ __device__ __forceinline__ void deposit_single(const HitKParams& kp, int32_t eve
   }
 }
 
-// ---- block max-scan of the tile's task-start marks ------------------------------
-template <int BLOCK, int HPT>
-__device__ __forceinline__ void owner_scan(int16_t* s_owner, int* s_wmax) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int v[HPT];
-  int run = 0;
-#pragma unroll
-  for (int k = 0; k < HPT; ++k) {
-    run = max(run, (int)s_owner[tid * HPT + k]);
-    v[k] = run;
-  }
-  int x = run;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x = max(x, y);
-  }
-  if (lane == 31) s_wmax[warp] = x;
-  __syncthreads();
-  int prefix = 0;
-  for (int w = 0; w < warp; ++w) prefix = max(prefix, s_wmax[w]);
-  int excl = __shfl_up_sync(0xffffffffu, x, 1);
-  if (lane == 0) excl = 0;
-  excl = max(excl, prefix);
-#pragma unroll
-  for (int k = 0; k < HPT; ++k) s_owner[tid * HPT + k] = (int16_t)max(v[k], excl);
-}
-
-// The uncertain hits of a warp step (need set, m = their ballot, non-zero):
-// queued for the FP64 recheck kernel as (task, hit in task); when the queue is
-// full the hit's cell is decided here in FP64, as the recheck kernel would.
-// Called by the whole warp; out of line, as it runs for well under one warp
-// step in a hundred.
+// The hits a warp has put off (one per lane, `have`: this lane has one): those
+// whose bin needs the search over the thresholds and those the staged map did
+// not certify.  Their cell comes from the search over the layer's regions, and
+// where that is not certain either the hit is queued for the FP64 recheck
+// kernel as (task, hit in task); when the queue is full its cell is decided
+// here in FP64, as the recheck kernel would.  Called by the whole warp; out of
+// line, as it runs once in some 50 warp steps (2 % of the hits, 32 at a time).
 template <int MODE, bool DBG>
-static __device__ __noinline__ void queue_uncertain(const HitKParams& kp, bool need, unsigned m, int64_t task,
-                                                    uint32_t hit, int32_t layer, float eta_c, float phi_c, uint4 x,
-                                                    int bin, int32_t ev, float Ehit, int32_t entry, int64_t dbg_h) {
+static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool have, uint2 th, float* s_v) {
   const WsDev& w = kp.w;
-  const int lane = threadIdx.x & 31;
-  unsigned long long base = 0;
-  const int l0 = __ffs(m) - 1;
-  if (lane == l0) base = atomicAdd((unsigned long long*)&w.sizes->n_recheck, (unsigned long long)__popc(m));
-  base = __shfl_sync(0xffffffffu, base, l0);
-  if (!need) return;
-  const unsigned long long pos = base + __popc(m & ((1u << lane) - 1u));
-  if (pos < (unsigned long long)w.recheck_cap) {
-    w.recheck[pos] = make_uint2((uint32_t)task, hit);
-    return;
+  TaskRec T{};
+  uint4 x = make_uint4(0u, 0u, 0u, 0u);
+  int bin = 0;
+  int32_t c = -1;
+  if (have) {
+    T = w.tasks[th.x];
+    x = philox4x32_10_rk(make_uint4(th.y, (uint32_t)T.layer() | (kPurposeHit << 16), (uint32_t)T.particle,
+                                    kp.first_event_lo + (uint32_t)T.event()),
+                         kp.rk);
+    bin = sample_bin(kp.p, (uint32_t)T.entry() * kNBins, x.x);
+    c = generic_cell(kp.g, kp.p, T, x, bin);
+    if (c < 0) {
+      const unsigned long long pos = atomicAdd((unsigned long long*)&w.sizes->n_recheck, 1ull);
+      if (pos < (unsigned long long)w.recheck_cap) {
+        w.recheck[pos] = th;
+      } else {
+        c = cell_fp64(kp.g, kp.p, T.layer(), T.eta_c, T.phi_c, x, bin);
+        atomicAdd((unsigned long long*)&w.sizes->n_inline, 1ull);
+        atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_RECHECK_SPILL);
+      }
+    }
+    if constexpr (DBG) {
+      const int64_t h = w.sizes->hit_base + w.th[th.x] + th.y;
+      if (h < kp.dbg_hit_cap) {
+        if (kp.dbg_hit_cell && c >= 0) kp.dbg_hit_cell[h] = c;
+        if (kp.dbg_hit_bin) kp.dbg_hit_bin[h] = (int16_t)bin;
+      }
+    }
   }
-  const int32_t c = cell_fp64(kp.g, kp.p, layer, eta_c, phi_c, x, bin);
-  deposit_single(kp, ev, Ehit, task, c, MODE, entry, bin);
-  atomicAdd((unsigned long long*)&w.sizes->n_inline, 1ull);
-  atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_RECHECK_SPILL);
-  if (DBG && kp.dbg_hit_cell && dbg_h < kp.dbg_hit_cap) kp.dbg_hit_cell[dbg_h] = c;
+  const bool ok = c >= 0;
+  const int64_t row = T.event() - kp.ev_lo;
+  const float Ehit = ok ? __fdiv_rn(T.El, (float)w.tn[th.x]) : 0.0f;
+  if constexpr (MODE == kModeGrad) {
+    const float v = ok ? __fmul_rn(Ehit, __ldg(kp.grad_in + row * kp.g.n_cells + c)) : 0.0f;
+    grad_warp(ok, ((uint32_t)T.entry() << 7) | (uint32_t)bin, v, s_v, kp);
+  } else if constexpr (MODE == kModeAtomic) {
+    if (ok) acc_add(w.acc + row * kp.g.acc_stride + c, Ehit);
+  } else {
+    // records as emit_records writes them, in slots of their own
+    const int lane = threadIdx.x & 31;
+    const uint32_t cg = (uint32_t)(row * kp.g.acc_stride + c);
+    const unsigned long long gkey = ((unsigned long long)cg << kp.key_task_bits) | th.x;
+    const unsigned peers = __ballot_sync(0xffffffffu, ok) & __match_any_sync(0xffffffffu, gkey);
+    const bool lead = ok && lane == __ffs(peers) - 1;
+    const unsigned lm = __ballot_sync(0xffffffffu, lead);
+    unsigned long long base = 0;
+    if (lane == 0 && lm) {
+      base = atomicAdd((unsigned long long*)&w.sizes->n_slots, (unsigned long long)__popc(lm));
+      atomicAdd((unsigned long long*)&w.sizes->n_records, (unsigned long long)__popc(lm));
+    }
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (lead) {
+      const int64_t slot = (int64_t)base + __popc(lm & ((1u << lane) - 1u));
+      if (slot < w.rec_cap) {
+        w.keys[slot] = (gkey << kRecordCountBits) | (unsigned long long)(__popc(peers) - 1);
+        atomicAdd(reinterpret_cast<uint32_t*>(w.acc) + cg, 1u);
+      } else {
+        atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_HIT_CAPACITY);
+      }
+    }
+  }
 }
 
-// Atomic mode asks for 10 CTAs of 128 threads per SM (48 registers): the
-// extra warps hide the guide-table loads; the other modes keep the
-// compiler's choice (a minimum of 0 CTAs is no constraint).  DBG: the
-// validation dumps of fcs_debug (a separate instantiation, so that the
-// production kernel carries none of their code).
-template <int BLOCK, int HPT, int MODE, bool DBG>
-__global__ void __launch_bounds__(BLOCK, MODE == kModeAtomic ? 1280 / BLOCK : 0) k_hits(const __grid_constant__ HitKParams kp) {
+// Every warp works by itself: it takes a ticket of consecutive hits and runs
+// through it in passes of up to NT tasks, one lane staging each, and the
+// pass's hits 32 at a time, two steps in flight.  No warp waits for another:
+// the long chains of dependent loads (a pass's task records, the hits put off)
+// stall one warp and the others of the SM fill in.
+//
+// What bounds it: instruction issue, at 0.6-0.7 of the slots, behind the
+// latency of the guide words (L2) that each step needs after its Philox block.
+// 64 pile-up events (86.8M hits), this kernel's time on the library's events:
+//   817 us  CTA tiles of 1024 hits with barriers, region tables in shared
+//           memory, a search of the thresholds and the regions in the loop
+//   768     one multiply-add per coordinate from staged tasks (1.7 fewer
+//           conversions and table loads per hit), task starts as bits
+//   729     neighbouring regions of one grid staged as one: 0.1 instead of
+//           0.5 % of the hits leave the map
+//   690     one 4-byte guide word, searches and uncertified hits put off to
+//           full warps (in the loop their branches took half the steps)
+//   598     a warp's own tickets and passes instead of CTA tiles
+//   571     two steps in flight; 9 CTAs of 128 threads per SM at 56 registers
+//           (10 at 48: 596, 8 at 64: 571, one step in flight: 600)
+// (Finishing the searches in the loop with two more loads: 610.  Without any
+// put-off hit, wrongly, it would be 500.)
+//
+// MIN CTAs per SM: the modes' best of 7 to 10.  DBG: the validation dumps of
+// fcs_debug (a separate instantiation, so that the production kernel carries
+// none of their code).
+constexpr int hits_min_ctas(int mode, int block) { return (mode == kModeAtomic ? 9 : 8) * 128 / block; }
+template <int BLOCK, int MODE, bool DBG>
+__global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(const __grid_constant__ HitKParams kp) {
   constexpr bool DET = MODE == kModeDet;
-  constexpr int TILE = BLOCK * HPT;
-  static_assert(TILE % kGranule == 0, "queue tiles must start on granules (the tile map's unit)");
-  static_assert(TILE <= 4096, "owner index and 32-bit match keys need TILE + 1 < 2^13");
+  constexpr int NW = BLOCK / 32;
+  constexpr int NT = BLOCK > 256 ? 24 : 32;  // staged tasks per warp (static shared memory holds 48 KB)
+  constexpr unsigned kAll = 0xffffffffu;
+  static_assert(kGuideCells == 2 * kNBins, "one base for guide cells and thresholds");
+  static_assert(kMaxTicket <= 1024, "a pass's task starts are 32 words, one per lane");
   __shared__ HitSmemTables tb;
-  __shared__ __align__(16) TileTask s_task[kSmemTasks];
-  __shared__ int16_t s_owner[TILE];
-  __shared__ int s_wmax[BLOCK / 32];
-  __shared__ uint32_t s_tile;
-  __shared__ float s_gv[MODE == kModeGrad ? BLOCK : 1];
+  __shared__ __align__(16) TileTask s_task[NW][NT];
+  __shared__ uint32_t s_start[NW][32];  // bit i of the pass: a task other than its first starts at hit i
+  __shared__ uint2 s_def[NW][96];       // hits put off (task, hit), fewer than 32 between rounds of two steps
+  __shared__ float s_gv[MODE == kModeGrad ? BLOCK : 1];  // gradient mode
   __shared__ unsigned long long s_recs;  // deterministic mode: records of this CTA
-  load_tables(tb, kp.g, kp.p);
-  for (int i = threadIdx.x; i < TILE; i += BLOCK) s_owner[i] = 0;
+  load_tables(tb, kp.p);
+  if (DET && threadIdx.x == 0) s_recs = 0;
+  __syncthreads();
   const WsDev& w = kp.w;
   const int64_t H = kp.static_tiles ? kp.h_hi : w.sizes->n_hits;
-  const int64_t T_last = kp.static_tiles ? (int64_t)kp.t_last : w.sizes->n_tasks - 1;
+  const int32_t T_end = kp.static_tiles ? kp.t_last + 1 : (int32_t)w.sizes->n_tasks;
   const int64_t hbase = kp.static_tiles ? kp.h_lo : 0;
   if (H > w.gmap_cap * (int64_t)kGranule) {  // the tile map is too small for the hits
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_HIT_CAPACITY);
     return;
   }
-  const uint32_t n_tiles = (uint32_t)((H - hbase + TILE - 1) / TILE);  // < 2^32: hits < 2^39
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const unsigned lanes_below = (1u << lane) - 1u;
-  const int64_t hit_dbg_base = DBG ? w.sizes->hit_base : 0;
+  const unsigned lanes_below = (1u << lane) - 1u, lanes_upto = lanes_below | (1u << lane);
+  // Hits per ticket: as many as leave each warp several tickets, since a pass
+  // of tasks costs as much as eight steps; small calls give each warp one.
+  const uint32_t n_warps = gridDim.x * NW;
+  const int64_t share = (H - hbase + n_warps - 1) / n_warps;  // hits per warp
+  uint32_t q = (uint32_t)kp.ticket;
+  if (q == 0) q = share > 4096 ? 1024u : share > 2048 ? 512u : share > 768 ? 256u : share > 256 || share <= 128 ? 128u : 256u;
+  const uint32_t n_tiles = (uint32_t)((H - hbase + q - 1) / q);  // < 2^32: hits < 2^39
   // accumulation rows (atomic, deterministic) or dL/dE_cell rows (gradient)
   const uint32_t row_stride = MODE == kModeGrad ? (uint32_t)kp.g.n_cells : (uint32_t)kp.g.acc_stride;
-  if (threadIdx.x == 0) {
-    s_tile = kp.static_tiles ? blockIdx.x : (uint32_t)atomicAdd(&w.sizes->queue, 1ull);
-    s_recs = 0;
-  }
-  __syncthreads();
-  uint32_t tile = s_tile;
+  const float r_max = __ldg(kp.p.r_edges + kNR);
   unsigned long long recs = 0;  // deterministic mode: this warp's records
   RecordChunk chunk;            //   and the slots it writes them to
-  while (tile < n_tiles) {
-    __syncthreads();  // everyone has read s_tile; s_owner is zero again
-    if (threadIdx.x == 0) s_tile = kp.static_tiles ? n_tiles : (uint32_t)atomicAdd(&w.sizes->queue, 1ull);
-    const int64_t h0 = hbase + (int64_t)tile * TILE;
-    const int hn = (int)min((int64_t)TILE, H - h0);  // hits in this tile
-    const int32_t t0 = kp.static_tiles ? kp.t_last : w.gmap[h0 / kGranule];
-    const int32_t t1 = (h0 + TILE < H && !kp.static_tiles) ? w.gmap[(h0 + TILE) / kGranule] : (int32_t)T_last;
-    const int nt = t1 - t0 + 1;
-    // (deterministic mode: the tile that holds a task's first hit writes the
-    // task's hit energy for the fold)
-    if (nt <= kSmemTasks) {
-      // stage the tile's tasks and mark where each starts
-      for (int j = threadIdx.x; j < nt; j += BLOCK) {
-        const TileTask q = make_tile_task(tb, w, t0 + j, h0, kp.first_event_lo, kp.ev_lo, row_stride);
-        const int64_t s = q.rel;
-        s_task[j] = q;
-        if (j > 0 && s < TILE) s_owner[s] = (int16_t)j;
-        if constexpr (DET) {
-          if (s >= 0 && s < TILE) w.tehit[t0 + j] = q.Ehit;
-        }
-      }
-    } else {
-      for (int j = threadIdx.x; j < nt; j += BLOCK) {
-        const int64_t s = w.th[t0 + j] - h0;
-        if (j > 0 && s < TILE) s_owner[s] = (int16_t)j;
-        if constexpr (DET) {
-          if (s >= 0 && s < TILE) w.tehit[t0 + j] = __fdiv_rn(w.tasks[t0 + j].El, (float)w.tn[t0 + j]);
-        }
-      }
+  int n_def = 0;                // this warp's hits in s_def
+  float* const s_v = MODE == kModeGrad ? s_gv + warp * 32 : nullptr;
+  // The first two thirds of the tickets go to the warps in turn, the rest
+  // through the queue (its counter serves a ticket in 2.2 ns), which evens out
+  // the warps' speeds; calls of many tickets a warp take all from the queue,
+  // whose stricter order keeps the rows and tables in flight few (64 events:
+  // 573 against 606 us; 7 events: 69 against 62 us).
+  const uint32_t n_turns = kp.static_tiles ? 1u : share > 8192 ? 0u : max(n_tiles / n_warps * 2u / 3u, 1u);
+  auto take = [&](uint32_t turn) {
+    uint32_t t = turn * n_warps + blockIdx.x * NW + warp;
+    if (turn >= n_turns) {
+      t = n_tiles;
+      if (!kp.static_tiles && lane == 0) t = n_turns * n_warps + (uint32_t)atomicAdd(&w.sizes->queue, 1ull);
     }
-    __syncthreads();
-    owner_scan<BLOCK, HPT>(s_owner, s_wmax);
-    __syncthreads();
-    // the hit loop, compiled once for staged tiles (the common case) and once
-    // for tiles with more tasks than the shared copy holds
-    auto hit_loop = [&](auto staged) {
-#pragma unroll 1
-      for (int k = 0; k < HPT; ++k) {
-        const int i = warp * 32 * HPT + k * 32 + lane;
-        const bool valid = i < hn;
-        const int tl = valid ? s_owner[i] : 0;
-        TileTask T;
-        if constexpr (decltype(staged)::value) {
-          T = s_task[tl];
-        } else {  // more tasks than the shared copy holds: read the record itself
-          T = make_tile_task(tb, w, t0 + tl, h0, kp.first_event_lo, kp.ev_lo, row_stride);
+    return t;  // of the lane 0
+  };
+  uint32_t turn = 0;
+  uint32_t tile = __shfl_sync(kAll, take(turn), 0);
+  while (tile < n_tiles) {
+    const uint32_t next = take(++turn);  // in flight during this ticket
+    int64_t h0 = hbase + (int64_t)tile * q;  // first hit of the pass
+    const int64_t h1 = min(h0 + (int64_t)q, H);
+    int32_t t0 = kp.static_tiles ? kp.t_last : w.gmap[h0 / kGranule];
+    while (h0 < h1) {
+      // stage the tasks t0 .. t0 + NT - 1 and mark where each starts
+      // (deterministic mode: the pass that holds a task's first hit writes the
+      // task's hit energy for the fold)
+      __syncwarp();
+      s_start[warp][lane] = 0;
+      __syncwarp();
+      int end = (int)(h1 - h0);  // hits of the pass
+      int after = end;           // where the lane's task ends
+      if (lane < NT && t0 + lane < T_end) {
+        const int64_t s64 = w.th[t0 + lane] - h0;
+        if (s64 < end) {
+          const TileTask t = make_tile_task(w, kp.g, t0 + lane, h0, kp.first_event_lo, kp.ev_lo, row_stride, r_max, kp.rk);
+          s_task[warp][lane] = t;
+          if (lane > 0) atomicOr(&s_start[warp][t.rel >> 5], 1u << (t.rel & 31));
+          if (lane == NT - 1) after = (int)min((int64_t)end, s64 + w.tn[t0 + lane]);
+          if constexpr (DET) {
+            if (t.rel >= 0) w.tehit[t0 + lane] = t.Ehit;
+          }
         }
-        const uint32_t hit = (uint32_t)(i - T.rel);
-        // the round keys come from the kernel parameters
-        const uint4 x = philox4x32_10_rk(make_uint4(hit, T.ctr_y, T.ctr_z, T.ctr_w), kp.rk);
-        const int bin = sample_bin(kp.p, T.entry, x.x);
-        const FastHit f = fast_cell(tb, T, x, bin);
-        const bool ok = valid && f.sure;
-        const bool need = valid && !f.sure;
+      }
+      end = __shfl_sync(kAll, after, NT - 1);
+      __syncwarp();
+      const uint32_t my_starts = s_start[warp][lane];
+      int tbase = 0;  // tasks that start in the steps before
+      // a step is 32 hits; its draw (task, random block, guide word) and its
+      // finish (bin, cell, deposit) are apart so that a second step's load is
+      // in flight before the first one's is used
+      struct Draw {
+        uint32_t x0, x1, x2, g, hit;
+        int tl;
+      };
+      auto draw = [&](int k) {
+        Draw d;
+        const uint32_t starts = __shfl_sync(kAll, my_starts, k);
+        d.tl = tbase + __popc(starts & lanes_upto);
+        tbase += __popc(starts);
+        const TileTask& T = s_task[warp][d.tl];
+        d.hit = (uint32_t)(k * 32 + lane - T.rel);
+        const uint4 x = hit_block(T, d.hit, kp.rk);
+        d.x0 = x.x;
+        d.x1 = x.y;
+        d.x2 = x.z;
+        d.g = guide_word(kp.p, T.gbase, x.x);
+        return d;
+      };
+      auto finish = [&](int k, const Draw& d) {
+        const TileTask& T = s_task[warp][d.tl];
+        const GuideBin gb = bin_in_cell(d.x0, d.g);
+        const int bin = gb.bin;
+        const FastHit f = fast_cell(tb, T, d.x1, d.x2, bin);
+        const bool valid = k * 32 + lane < end;
+        const bool ok = valid && f.sure && !gb.search;
         if constexpr (MODE == kModeGrad) {
           // dL/dE_cell of the hit's cell times its energy, summed per (entry, bin)
-          const float v = ok ? __fmul_rn(T.Ehit, __ldg(kp.grad_in + T.row_off + f.cell)) : 0.0f;
-          grad_warp(ok, ((uint32_t)T.entry << 7) | (uint32_t)bin, v, s_gv + warp * 32, kp);
+          const float v = ok ? __fmul_rn(T.Ehit, __ldg(kp.grad_in + f.cell)) : 0.0f;
+          grad_warp(ok, T.gbase | (uint32_t)bin, v, s_v, kp);
         } else if constexpr (!DET) {
-          // (cell, task-in-tile) identifies (address, hit energy): 19 + 13 bits
-          const unsigned m = __ballot_sync(0xffffffffu, ok);
-          if (ok) {
-            const unsigned peers = kp.key32 ? __match_any_sync(m, ((uint32_t)f.cell << 13) | (uint32_t)tl)
-                                            : __match_any_sync(m, ((unsigned long long)(uint32_t)tl << 32) |
-                                                                      (uint32_t)f.cell);
-            if ((peers & lanes_below) == 0u)  // the group's first lane deposits
-              acc_add(w.acc + T.row_off + f.cell, __fmul_rn((float)__popc(peers), T.Ehit));
-          }
+          // the low 27 bits of the row offset + cell tell a task's cells apart
+          // (n_cells < 2^27): with the task in the pass they identify (address, hit energy)
+          const unsigned m = __ballot_sync(kAll, ok);
+          const unsigned peers =
+              m & (kp.key32 ? __match_any_sync(kAll, (f.cell << 5) | (uint32_t)d.tl)
+                            : __match_any_sync(kAll, ((unsigned long long)(uint32_t)d.tl << 32) | f.cell));
+          if (ok && (peers & lanes_below) == 0u)  // the group's first lane deposits
+            acc_add(w.acc + f.cell, __fmul_rn((float)__popc(peers), T.Ehit));
         } else {
-          const uint32_t cg = T.row_off + (uint32_t)f.cell;
-          const unsigned long long gkey = ((unsigned long long)cg << kp.key_task_bits) | (unsigned long long)(t0 + tl);
-          recs += emit_records(ok, gkey, cg, chunk, w);
+          const unsigned long long gkey =
+              ((unsigned long long)f.cell << kp.key_task_bits) | (unsigned long long)(t0 + d.tl);
+          recs += emit_records(ok, gkey, f.cell, chunk, w);
         }
-        // queue the uncertain hits for the FP64 recheck
-        const unsigned m = __ballot_sync(0xffffffffu, need);
-        if (m)
-          queue_uncertain<MODE, DBG>(kp, need, m, t0 + tl, hit, (int32_t)(T.lay & 0xFF), T.eta_c, T.phi_c, x, bin,
-                                     (int32_t)(T.ctr_w - kp.first_event_lo), T.Ehit, T.entry, hit_dbg_base + h0 + i);
         if constexpr (DBG) {
-          const int64_t h = hit_dbg_base + h0 + i;
-          if (valid && h < kp.dbg_hit_cap) {
-            if (kp.dbg_hit_cell && f.sure) kp.dbg_hit_cell[h] = f.cell;
+          const int64_t h = w.sizes->hit_base + h0 + k * 32 + lane;
+          if (ok && h < kp.dbg_hit_cap) {
+            if (kp.dbg_hit_cell)
+              kp.dbg_hit_cell[h] =
+                  (int32_t)(f.cell - (uint32_t)(w.tasks[t0 + d.tl].event() - kp.ev_lo) * row_stride);
             if (kp.dbg_hit_bin) kp.dbg_hit_bin[h] = (int16_t)bin;
           }
         }
-        s_owner[i] = 0;  // ready for the next tile (each slot is read and reset by one thread)
+        const unsigned md = __ballot_sync(kAll, valid && !ok);
+        if (md) {  // put off
+          if ((md >> lane) & 1u)
+            s_def[warp][n_def + __popc(md & lanes_below)] = make_uint2((uint32_t)(t0 + d.tl), d.hit);
+          n_def += __popc(md);
+        }
+      };
+#pragma unroll 1
+      for (int k = 0; k * 32 < end; k += 2) {
+        const Draw d0 = draw(k);
+        if ((k + 1) * 32 < end) {
+          const Draw d1 = draw(k + 1);
+          finish(k, d0);
+          finish(k + 1, d1);
+        } else {
+          finish(k, d0);
+        }
+        if (n_def >= 32) {  // 32 put-off hits go through the search
+          __syncwarp();
+          do {
+            n_def -= 32;
+            deferred_hits<MODE, DBG>(kp, true, s_def[warp][n_def + lane], s_v);
+          } while (n_def >= 32);
+          __syncwarp();
+        }
       }
-    };
-    if (nt <= kSmemTasks) hit_loop(std::true_type{});
-    else hit_loop(std::false_type{});
-    __syncthreads();  // the tile's shared data is dead; s_tile holds the next tile
-    tile = s_tile;
+      h0 += end;
+      t0 += NT;
+    }
+    tile = __shfl_sync(kAll, next, 0);
   }
+  __syncwarp();
+  if (n_def) deferred_hits<MODE, DBG>(kp, lane < n_def, s_def[warp][lane], s_v);
   if constexpr (DET) {
     close_records(chunk, w);
     if (lane == 0 && recs) atomicAdd(&s_recs, recs);
@@ -614,9 +756,9 @@ __global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ HitKPar
     const uint4 x = philox4x32_10(
         make_uint4(q.y, (uint32_t)layer | (kPurposeHit << 16), (uint32_t)T.particle, kp.first_event_lo + (uint32_t)event),
         kp.k0, kp.k1);
-    const int bin = sample_bin(kp.p, T.entry, x.x);
+    const int bin = sample_bin(kp.p, (uint32_t)T.entry() * kNBins, x.x);
     const int32_t c = cell_fp64(kp.g, kp.p, layer, T.eta_c, T.phi_c, x, bin);
-    deposit_single(kp, event, __fdiv_rn(T.El, (float)w.tn[q.x]), q.x, c, MODE, T.entry, bin);
+    deposit_single(kp, event, __fdiv_rn(T.El, (float)w.tn[q.x]), q.x, c, MODE, T.entry(), bin);
     const int64_t h = hit_dbg_base + hb + q.y;
     if (kp.dbg_hit_cell && h < kp.dbg_hit_cap) kp.dbg_hit_cell[h] = c;
   }

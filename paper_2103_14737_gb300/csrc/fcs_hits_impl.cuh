@@ -1,5 +1,4 @@
-// fcs_hits_impl.cuh - launch dispatch of the hit kernel over the tuned
-// (threads per block, hits per thread) shapes; included by the atomic-mode,
+// fcs_hits_impl.cuh - launch dispatch of the hit kernel over its block sizes; included by the atomic-mode,
 // deterministic-mode and gradient-mode translation units.
 #pragma once
 
@@ -19,7 +18,7 @@ static inline HitKParams make_hit_params(const GeoDev& g, const ParamDev& p, WsD
   kp.k1 = k1;
   kp.first_event_lo = (uint32_t)first_event;
   kp.key_task_bits = key_task_bits;
-  kp.key32 = g.n_cells < (1 << 19) ? 1 : 0;
+  kp.key32 = g.n_cells < (1 << 27) ? 1 : 0;
   kp.dbg_hit_cell = dbg ? dbg->hit_cell : nullptr;
   kp.dbg_hit_bin = dbg ? dbg->hit_bin : nullptr;
   kp.dbg_hit_cap = dbg ? dbg->hit_capacity : 0;
@@ -27,43 +26,47 @@ static inline HitKParams make_hit_params(const GeoDev& g, const ParamDev& p, WsD
   return kp;
 }
 
-template <int BLOCK, int HPT, int MODE, bool DBG>
+template <int BLOCK, int MODE, bool DBG>
 static cudaError_t launch_hits_kernel(const HitKParams& kp, const Launch& L) {
   static int occ = -1;  // resident CTAs per SM of this instantiation
   if (occ < 0) {
     int o = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_hits<BLOCK, HPT, MODE, DBG>, BLOCK, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_hits<BLOCK, MODE, DBG>, BLOCK, 0);
     if (e != cudaSuccess) return e;
     occ = o < 1 ? 1 : o;
   }
   int64_t grid = (int64_t)L.num_sms * occ;
   if (kp.static_tiles) {
-    constexpr int64_t TILE = (int64_t)BLOCK * HPT;
-    grid = (kp.h_hi - kp.h_lo + TILE - 1) / TILE;
+    const int64_t per_cta = (int64_t)kp.ticket * (BLOCK / 32);
+    grid = (kp.h_hi - kp.h_lo + per_cta - 1) / per_cta;
     if (grid <= 0) return cudaSuccess;
   }
-  k_hits<BLOCK, HPT, MODE, DBG><<<(unsigned)grid, BLOCK, 0, L.s>>>(kp);
+  k_hits<BLOCK, MODE, DBG><<<(unsigned)grid, BLOCK, 0, L.s>>>(kp);
   return cudaGetLastError();
 }
 
 // The validation dumps run in their own instantiation (no gradient-mode dumps).
-template <int BLOCK, int HPT, int MODE>
-static cudaError_t launch_hits_shape(const HitKParams& kp, const Launch& L) {
+template <int BLOCK, int MODE>
+static cudaError_t launch_hits_block(const HitKParams& kp, const Launch& L) {
   if constexpr (MODE != kModeGrad) {
-    if (kp.dbg_hit_cell || kp.dbg_hit_bin) return launch_hits_kernel<BLOCK, HPT, MODE, true>(kp, L);
+    if (kp.dbg_hit_cell || kp.dbg_hit_bin) return launch_hits_kernel<BLOCK, MODE, true>(kp, L);
   }
-  return launch_hits_kernel<BLOCK, HPT, MODE, false>(kp, L);
+  return launch_hits_kernel<BLOCK, MODE, false>(kp, L);
 }
 
+// hc.hpt sets the queue's tickets, kGranule hits per unit (at most
+// kMaxTicket); 0 leaves them to the kernel, which knows the call's hits.
 template <int MODE>
-cudaError_t launch_hits_t(const HitKParams& kp, const HitCfg& hc, const Launch& L) {
-#define FCS_HIT_CASE(B, H) \
-  if (hc.block == B && hc.hpt == H) return launch_hits_shape<B, H, MODE>(kp, L);
-  FCS_HIT_CASE(128, 1) FCS_HIT_CASE(128, 2) FCS_HIT_CASE(128, 4) FCS_HIT_CASE(128, 8)
-  FCS_HIT_CASE(256, 1) FCS_HIT_CASE(256, 2) FCS_HIT_CASE(256, 4) FCS_HIT_CASE(256, 8)
-  FCS_HIT_CASE(512, 1) FCS_HIT_CASE(512, 2) FCS_HIT_CASE(512, 4) FCS_HIT_CASE(512, 8)
-#undef FCS_HIT_CASE
-  return cudaErrorInvalidValue;
+cudaError_t launch_hits_t(const HitKParams& kp0, const HitCfg& hc, const Launch& L) {
+  HitKParams kp = kp0;
+  kp.ticket = std::min(hc.hpt * kGranule, kMaxTicket);
+  if (kp.static_tiles && !kp.ticket) kp.ticket = 2 * kGranule;
+  switch (hc.block) {
+    case 128: return launch_hits_block<128, MODE>(kp, L);
+    case 256: return launch_hits_block<256, MODE>(kp, L);
+    case 512: return launch_hits_block<512, MODE>(kp, L);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 template <int MODE>

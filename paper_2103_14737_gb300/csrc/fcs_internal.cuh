@@ -16,7 +16,7 @@ constexpr int kMaxRegions = 256;
 constexpr int kNBins = 128;      // 16 r-bins x 8 alpha-bins
 constexpr int kNR = 16;
 constexpr int kNA = 8;
-constexpr int kGuideCells = 128; // guide cells per histogram (top 7 bits of word 0)
+constexpr int kGuideCells = 256; // guide cells per histogram (top 8 bits of word 0)
 constexpr int kRecordChunk = 256;  // deterministic mode: record slots a warp takes at a time
 constexpr int64_t kRecordSlack = 1 << 22;  // slots beyond the hits: the warps' partly filled chunks
 constexpr int kGranule = 128;    // hits per granule of the tile -> task map (divides every tile)
@@ -30,7 +30,7 @@ constexpr int kLfactEntries = 8192;  // log k! table for the FP32 Poisson test (
 // range); the hit energy is fl32(El / n) (Listing 1: float Ehit = E(layer) /
 // nhit), formed where a kernel needs it.
 struct __align__(16) TaskRec {
-  int32_t entry;       // parametrisation entry including the layer
+  uint32_t entry_reg;  // parametrisation entry including the layer (24 bits) | home region << 24
   float El;            // layer energy fl32(E f_l), MeV
   float eta_c, phi_c;
   float s_eta, s_phi;  // FP32 scale factors of the (r, alpha) -> (eta, phi) map
@@ -38,23 +38,35 @@ struct __align__(16) TaskRec {
   uint32_t ev_layer;   // batch-local event << 8 | layer
   __device__ __forceinline__ int32_t event() const { return (int32_t)(ev_layer >> 8); }
   __device__ __forceinline__ int32_t layer() const { return (int32_t)(ev_layer & 0xFFu); }
+  __device__ __forceinline__ int32_t entry() const { return (int32_t)(entry_reg & 0xFFFFFFu); }
+  // the region of the layer that owns eta_c (up to the rounding of its FP32 boundary)
+  __device__ __forceinline__ int32_t region() const { return (int32_t)(entry_reg >> 24); }
 };
 static_assert(sizeof(TaskRec) == 32, "TaskRec layout");
 constexpr int32_t kMaxEventsPerCall = 1 << 24;  // batch-local events fit the record's 24 bits
 
-// FP32 view of a region for the fast path (shared-memory staged): the scaled
-// indices are te = eta inv_deta + ek and tp = phi inv_dphi + pk, one FMA each,
-// and the constant parts of their error bounds come with the region.
+// FP32 view of a region.  Fast path (fcs_hits.cuh: make_tile_task), for the
+// region and the neighbours that continue its grid (equal granularity, edges
+// that meet: fcs_load_geometry) as one grid: a hit's eta index minus 1/2 is
+// eta inv_deta + ekh, clamped to [lo, hi], its phi index minus 1/2 phi inv_dphi
+// + pkh.  Where the layer has no region below the grid, lo = 0 (every hit below
+// belongs to its first cell); where it has one, lo = -1/2, the grid's edge, at
+// which no hit is certified (and likewise hi = n_eta - 1 or n_eta - 1/2 above).
+// The other fields serve the search over the layer's regions (generic_cell).
 struct __align__(16) RegionF {
-  float ek, inv_deta;  // -eta_lo / deta (FP32 of the FP64 quotient), 1 / deta
-  float pk, inv_dphi;  // -phi_lo / dphi, 1 / dphi
-  float n_eta_hf;      // n_eta - 1/2: the scaled eta index is clamped to [1/2, n_eta - 1/2]
-  float ce;            // |ek| 2^-23 + 2^-22: eta-index bound beyond the position's and |te| 2^-21
-  float cp;            // |pk| 2^-23 + 2^-22: phi-index bound beyond the position's and |tp| 2^-21
-  int32_t n_phi, cell_off;
-  int32_t pad[3];
+  float ekh, inv_deta;  // -eta_lo / deta - 1/2 (FP32 of the FP64 value), 1 / deta
+  float pkh, inv_dphi;  // -phi_lo / dphi - 1/2, 1 / dphi
+  float lo, hi;
+  float n_eta;          // eta cells of the grid
+  float fast_off;       // 1 where a neighbour's boundary lies inside the grid (no hit is certified), else 0
+  int32_t n_phi, fast_cell;  // the grid's first cell
+  float ek, pk;         // -eta_lo / deta, -phi_lo / dphi
+  float n_eta_hf;       // n_eta - 1/2: the scaled eta index is clamped to [1/2, n_eta - 1/2]
+  float ce;             // |ek| 2^-23 + 2^-22: eta-index bound beyond the position's and |te| 2^-21
+  float cp;             // |pk| 2^-23 + 2^-22: phi-index bound beyond the position's and |tp| 2^-21
+  int32_t cell_off;
 };
-static_assert(sizeof(RegionF) == 48, "RegionF layout");
+static_assert(sizeof(RegionF) == 64, "RegionF layout");
 
 // Device geometry (all pointers device memory owned by fcs_geo).
 struct GeoDev {
@@ -66,6 +78,9 @@ struct GeoDev {
   const double* dphi;
   const double* split;   // split[r] for r > layer's first region
   const float* split32;  // [n_regions] FP32 of split (the lower ownership boundary); -inf for a layer's first
+  const float4* grids;   // [n_layers] the boundaries (FP32) between the layer's grids (RegionF) x, y, z (+inf where
+                         // there are fewer) and, in w, a region of each, 8 bits apiece; x is NaN for a layer of
+                         // more than four grids
   const int32_t* n_eta;
   const int32_t* n_phi;
   const int32_t* cell_off;
@@ -89,8 +104,8 @@ struct ParamDev {
   const float* shape_w;  // [n_entries][128] shape weights (the gradient's likelihood ratios)
   const float* mhe;      // [n_entries]
   const uint32_t* thr;   // [n_entries][128] inverse-CDF thresholds
-  const uint2* guide;    // [n_entries][128] packed guide cells (fcs_params.cu: thresholds T[lo], T[lo + 1]
-                         // as offsets within the cell, lo, hi - lo)
+  const uint32_t* guide; // [n_entries][256] packed guide cells (fcs_params.cu: threshold T[lo] as an offset
+                         // within the cell, lo, whether the cell holds more)
   const float* r_edges;  // [17]
   const float* a_edges;  // [9]
 };
@@ -146,14 +161,15 @@ struct WsDev {
 
 // Philox4x32-10 (Salmon et al., SC'11): published multipliers and Weyl
 // constants; counter c, key (k0, k1).
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+__device__ __forceinline__ uint4 philox_round(uint4 c, uint32_t k0, uint32_t k1) {
+  return make_uint4(__umulhi(kPhiloxM1, c.z) ^ c.y ^ k0, kPhiloxM1 * c.z, __umulhi(kPhiloxM0, c.x) ^ c.w ^ k1,
+                    kPhiloxM0 * c.x);
+}
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1) {
 #pragma unroll
   for (int i = 0; i < 10; ++i) {
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo0 = 0xD2511F53u * c.x;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z;
-    c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+    c = philox_round(c, k0, k1);
     k0 += 0x9E3779B9u;
     k1 += 0xBB67AE85u;
   }
@@ -175,13 +191,7 @@ __host__ __device__ inline PhiloxRoundKeys philox_round_keys(uint32_t k0, uint32
 }
 __device__ __forceinline__ uint4 philox4x32_10_rk(uint4 c, const PhiloxRoundKeys& rk) {
 #pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    const uint32_t hi0 = __umulhi(0xD2511F53u, c.x);
-    const uint32_t lo0 = 0xD2511F53u * c.x;
-    const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z);
-    const uint32_t lo1 = 0xCD9E8D57u * c.z;
-    c = make_uint4(hi1 ^ c.y ^ rk.k[2 * i], lo1, hi0 ^ c.w ^ rk.k[2 * i + 1], lo0);
-  }
+  for (int i = 0; i < 10; ++i) c = philox_round(c, rk.k[2 * i], rk.k[2 * i + 1]);
   return c;
 }
 
@@ -249,8 +259,11 @@ struct Launch {
 };
 
 // fcs_params.cu
-cudaError_t launch_build_tables(const float* shape_w, int n_entries, uint32_t* thr, uint2* guide,
-                                int32_t* bad, cudaStream_t s);
+// Thresholds and guide cells of the entries with frac > 0: all of them (all
+// != 0), or those whose flag in built [n_entries] is not set; sets the flags.
+// list [n_entries] and n_list: device scratch.
+cudaError_t launch_build_tables(const float* frac, const float* shape_w, int n_entries, int all, uint8_t* built,
+                                int32_t* list, int32_t* n_list, uint32_t* thr, uint32_t* guide, cudaStream_t s);
 
 // fcs_scan.cu: exclusive scan of n int64 values (n on the host or device),
 // one pass.  The state (ticket, done count, one status word per tile) is zero
@@ -314,7 +327,6 @@ cudaError_t launch_hits_task(const GeoDev& g, const ParamDev& p, WsDev w, int32_
 cudaError_t launch_recheck(const GeoDev& g, const ParamDev& p, WsDev w, int32_t ev_lo, uint32_t k0,
                            uint32_t k1, int64_t first_event, int det, int key_task_bits,
                            const fcs_debug* dbg, const Launch& L);
-int hits_max_smem_tasks();
 
 // fcs_grad.cu: the adjoint of the hit loop.  grad_in: dL/dE_cell rows of the
 // range (row stride n_cells); grad_acc: FP64 [n_entries][128] scores;

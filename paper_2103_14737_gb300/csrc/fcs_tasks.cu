@@ -530,6 +530,20 @@ __device__ __forceinline__ void ptrs_round(WarpQueue& q, const WsDev& w, const P
   warp_push(valid && k == -2, d.t, (unsigned long long*)&w.sizes->n_pdefer_ptrs, w.pdefer, true, w.pdefer_cap);
 }
 
+// The region of layer l (a member of its grid, GeoDev::grids) that owns eta.
+// Layers of up to four grids, all but odd geometries, take one 16-byte load.
+__device__ __forceinline__ uint32_t home_region(const GeoDev& g, int l, float eta) {
+  const float4 s = __ldg(g.grids + l);
+  if (s.x == s.x) {
+    const int n = (eta >= s.x ? 8 : 0) + (eta >= s.y ? 8 : 0) + (eta >= s.z ? 8 : 0);
+    return (__float_as_uint(s.w) >> n) & 0xFFu;
+  }
+  const int rb = __ldg(g.lrb + l), re = __ldg(g.lrb + l + 1);
+  int home = rb;
+  for (int q = rb + 1; q < re; ++q) home = eta >= __ldg(g.split32 + q) ? q : home;
+  return (uint32_t)home;
+}
+
 __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g, const ParamDev p,
                                                                  const fcs_particles parts, int32_t ev_lo, WsDev w,
                                                                  PhiloxRoundKeys rk, uint32_t first_event_lo) {
@@ -601,7 +615,7 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g,
         const int64_t e = (int64_t)entry * NL + l;
         const float El = __fmul_rn(oE, __ldg(p.frac + e));
         TaskRec r;
-        r.entry = (int32_t)e;
+        r.entry_reg = (uint32_t)e | (home_region(g, l, oeta) << 24);
         r.El = El;
         r.eta_c = oeta;
         r.phi_c = ophi;
@@ -651,7 +665,7 @@ __global__ void __launch_bounds__(128) k_task_poisson64(WsDev w, const float* mh
     const TaskRec& r = w.tasks[t];
     const uint32_t layer = (uint32_t)r.layer(), particle = (uint32_t)r.particle;
     const uint32_t event = first_event_lo + (uint32_t)r.event();
-    const float mu = __fdiv_rn(r.El, __ldg(mhe + r.entry));
+    const float mu = __fdiv_rn(r.El, __ldg(mhe + r.entry()));
     int64_t k = inv ? poisson_draw((double)mu, layer, particle, event, rk.k[0], rk.k[1], lfact64, n_lfact, 0u)
                     : ptrs_resume(mu, layer, particle, event, rk.k[0], rk.k[1], rk, lfact, lfact64, n_lfact,
                                   (uint32_t)w.tn[t]);

@@ -1,0 +1,73 @@
+"""GPU tests of the hit kernel's passes and of the table build: tickets of
+every size over tasks of one hit (many passes of 32 tasks to a ticket) and of
+thousands (a pass of one task), and tables rebuilt by an update of the weights
+or the fractions alone.  Deterministic mode is bit-exact against the oracle's
+canonical fold, so every cell checks every hit's bin and cell."""
+import dataclasses
+
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_2103_14737_gb300 import fcs, synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+@pytest.mark.parametrize("hit_E", [(2.0e4, 1.0e5), (0.05, 0.2)])  # about one hit a task; up to thousands
+def test_tickets(geo, ogeo, hit_E):
+    prm = synth.params(geo, mean_hit_range=hit_E)
+    parts = synth.ttbar_like(4, 2, n=150 if hit_E[0] > 1.0 else 8)
+    ref = O.simulate(ogeo, O.OracleParams(prm), parts, seed=9)
+    s = fcs.Simulator(geo, prm)
+    try:
+        d = s.to_device(parts)
+        for hpt in (0, 1, 2, 4, 8):
+            for block in (0, 256, 512):
+                got = s.simulate(d, 9, mode=fcs.MODE_DETERMINISTIC, dense=True, hits_per_thread=hpt, block=block)
+                assert got["stats"]["n_hits"] == ref.n_hits
+                assert np.array_equal(got["cells"].cpu().numpy().view(np.uint32), ref.cells_canon.view(np.uint32)), (hpt, block)
+                atom = s.simulate(d, 9, dense=True, hits_per_thread=hpt, block=block)["cells"].cpu().numpy()
+                assert (np.abs(atom - ref.cells64) <= 1e-5 * np.abs(ref.cells64) + 1e-3).all()
+    finally:
+        s.close()
+
+
+def test_table_updates(geo, prm, ogeo):
+    """Weights updated while some fractions are 0, then the fractions alone:
+    the entries that come alive have tables of the present weights."""
+    parts = synth.ttbar_like(3, 1)
+    rng = np.random.default_rng(2)
+    off = rng.random(prm.frac.shape) < 0.5
+    off[..., 0] = False
+    off[..., 4] = False
+    frac0 = np.where(off, 0.0, prm.frac).astype(np.float32)
+    w1 = (prm.shape_w * (0.5 + rng.random(prm.shape_w.shape))).astype(np.float32)
+    s = fcs.Simulator(geo, dataclasses.replace(prm, frac=frac0))
+    try:
+        d = s.to_device(parts)
+
+        def check(p):
+            ref = O.simulate(ogeo, O.OracleParams(p), parts, 5)
+            det = s.simulate(d, 5, mode=fcs.MODE_DETERMINISTIC, dense=True)["cells"].cpu().numpy()
+            assert np.array_equal(det.view(np.uint32), ref.cells_canon.view(np.uint32))
+
+        def dev(a):
+            return torch.as_tensor(np.ascontiguousarray(a), device="cuda").reshape(-1)
+
+        check(dataclasses.replace(prm, frac=frac0))
+        s.update_params(frac=dev(prm.frac))  # entries that were off at the load
+        check(prm)
+        s.update_params(frac=dev(frac0), shape_w=dev(w1))
+        check(dataclasses.replace(prm, frac=frac0, shape_w=w1))
+        s.update_params(frac=dev(prm.frac))  # entries that were off when the weights came
+        check(dataclasses.replace(prm, shape_w=w1))
+    finally:
+        s.close()
