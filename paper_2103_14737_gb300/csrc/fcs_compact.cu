@@ -14,144 +14,191 @@ namespace fcs {
 namespace {
 
 constexpr int kCThreads = 256;
-constexpr int kCItems = 16;  // eight 16-byte loads of FP64 cells per thread (rows are padded to 64 cells)
-constexpr int kCVec = kCItems / 2;
-constexpr int kChunk = kCThreads * kCItems;
-constexpr int kCtasPerSm = 4;  // resident: 54 registers x 256 threads each
+constexpr int kCWarps = kCThreads / 32;
+constexpr int kCRows = 8;               // 64-cell rows of a warp's share (rows are padded to 64 cells)
+constexpr int kShare = 64 * kCRows;
+constexpr int kChunk = kCWarps * kShare;  // 4096 cells
+constexpr int kCtasPerSm = 4;
 
 // A row value is a hit cell when it is not +-0 (an integer test, off the FP64 pipe).
 __device__ __forceinline__ bool acc_nonzero(double d) {
   return ((unsigned long long)__double_as_longlong(d) << 1) != 0ull;
 }
 
-// One pass: CTAs take chunks in ticket order; a chunk counts its hit cells,
-// publishes the count, looks back for the count of the chunks before it (the
-// first chunk starts at *total_dst, the call's running output size) and
-// writes its pairs; the last chunk leaves the new total in *total_dst.  The
-// last CTA to finish resets the ticket and the status words.
-__global__ void __launch_bounds__(kCThreads) k_compact_one(
-    double* __restrict__ acc, int32_t n_cells, int32_t stride, int32_t cpr, int64_t n_chunks, int32_t ev_lo,
-    uint64_t* __restrict__ state, int64_t cap_tiles, uint32_t* flags, int64_t* total_dst, float* __restrict__ cells_out,
-    int32_t* __restrict__ cell_ids, float* __restrict__ cell_E, int64_t* __restrict__ event_offsets_out,
-    int64_t capacity) {
-  __shared__ int s_w[kCThreads / 32];
-  __shared__ int32_t s_id[kChunk];
-  __shared__ float s_E[kChunk];
-  __shared__ int s_total;
-  __shared__ int64_t s_base;
+struct CompactArgs {
+  double* acc;
+  int32_t n_cells, stride, cpr, ev_lo;
+  int32_t one_run;
+  int64_t n_chunks;
+  uint64_t* state;
+  int64_t cap_tiles;
+  uint32_t* flags;
+  int64_t* total_dst;
+  float* cells_out;
+  int32_t* cell_ids;
+  float* cell_E;
+  int64_t* event_offsets_out;
+  int64_t capacity;
+};
+
+// One pass over the chunks: CTAs take them in ticket order; a chunk packs its
+// hit cells into shared memory as it reads them, publishes their count, looks
+// back for the count of the chunks before it (the first chunk starts at
+// *total_dst, the call's running output size) and writes its pairs; the last
+// chunk leaves the new total in *total_dst.  The last CTA to finish resets the
+// ticket and the status words.  A chunk's ticket is taken when the chunk before
+// it is written: a chunk held while its CTA still looks back publishes nothing,
+// and every look-back behind it waits (1024 events: 3270 us).
+//
+// Bound by memory (the rows in, the pairs out, the zeros) and by the look-backs:
+// 32 chunks in half a microsecond.  A warp takes 512 consecutive cells, 64 to
+// an instruction, 16 bytes a lane, all eight rows in flight at once; places in
+// the output come from ballots.  Compaction of 500 single electrons (753 MB of
+// nearly empty rows), 64 and 1024 pile-up events (1.5 GB of rows, 95M pairs):
+//   387, 78 and 960 us   each lane 16 consecutive cells, places by a block scan
+//   275, 65 and 795      here
+//   248, 74 and 866      8192-cell chunks (before the warps wrote by themselves)
+//   369, 100 and 1356    chunks by bulk copy into shared memory, three in
+//                        flight a CTA (its tickets are held)
+// DENSE: also the dense rows.  PAIRS: the pairs are wanted (else their number).
+template <bool DENSE, bool PAIRS>
+__global__ void __launch_bounds__(kCThreads, kCtasPerSm) k_compact_one(const CompactArgs A) {
+  __shared__ float s_E[PAIRS ? kChunk : 1];
+  __shared__ uint16_t s_at[PAIRS ? kChunk : 1];  // place in the chunk
+  __shared__ int s_w[kCWarps];
   __shared__ unsigned long long s_ticket;
+  __shared__ int64_t s_base;
   __shared__ int s_last;
-  unsigned long long* ticket = reinterpret_cast<unsigned long long*>(state);
+  unsigned long long* ticket = reinterpret_cast<unsigned long long*>(A.state);
   unsigned long long* done = ticket + 1;
-  uint64_t* status = state + 2;
-  int64_t n_t = n_chunks;
-  if (n_t > cap_tiles) {  // the workspace sizes the state for its chunks: never
-    if (threadIdx.x == 0) atomicOr(flags, (uint32_t)FCS_FLAG_WAIT_TIMEOUT);
+  uint64_t* status = A.state + 2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  int64_t n_t = A.n_chunks;
+  if (n_t > A.cap_tiles) {  // the workspace sizes the state for its chunks: never
+    if (tid == 0) atomicOr(A.flags, (uint32_t)FCS_FLAG_WAIT_TIMEOUT);
     n_t = 0;
   }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   while (true) {
-    if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1ull);
+    if (tid == 0) s_ticket = atomicAdd(ticket, 1ull);
     __syncthreads();
     const int64_t t = (int64_t)s_ticket;
     if (t >= n_t) break;
-    const int chunk = (int)(t % cpr), row = (int)(t / cpr);
-    const int64_t c0 = (int64_t)chunk * kChunk + threadIdx.x * kCItems;
-    double2* src = reinterpret_cast<double2*>(acc + (int64_t)row * stride + c0);
-    float v[kCItems];
-    unsigned mask = 0;
+    const int64_t row = t / A.cpr;
+    const int cc = (int)(t % A.cpr) * kChunk;  // the chunk's first cell in its row
+    const int c0 = cc + warp * kShare;         // the warp's
+    const int rows = min(kCRows, max(0, (A.stride - c0) / 64));
+    double2* const src = reinterpret_cast<double2*>(A.acc + row * A.stride + c0) + lane;
+    float* const dense = DENSE ? A.cells_out + (int64_t)(A.ev_lo + row) * A.n_cells : nullptr;
+    int n = 0;  // the warp's hit cells
+    double2 v[kCRows];
 #pragma unroll
-    for (int k = 0; k < kCItems; ++k) v[k] = 0.0f;
-    if (c0 < n_cells) {
-      double2 a[kCVec];
+    for (int j = 0; j < kCRows; ++j) v[j] = j < rows ? src[32 * j] : make_double2(0.0, 0.0);
 #pragma unroll
-      for (int q = 0; q < kCVec; ++q) a[q] = src[q];
-      const double2 z = make_double2(0.0, 0.0);
-#pragma unroll
-      for (int q = 0; q < kCVec; ++q) {
-        if (c0 + 2 * q < n_cells && acc_nonzero(a[q].x)) {
-          mask |= 1u << (2 * q);
-          v[2 * q] = acc_to_f32(a[q].x);
+    for (int j = 0; j < kCRows; ++j) {
+      const bool nx = acc_nonzero(v[j].x), ny = acc_nonzero(v[j].y);
+      const unsigned mx = __ballot_sync(0xffffffffu, nx), my = __ballot_sync(0xffffffffu, ny);
+      float fx = 0.0f, fy = 0.0f;
+      if (mx | my) {
+        if (nx || ny) src[32 * j] = make_double2(0.0, 0.0);  // re-zero what is not zero
+        if (DENSE || PAIRS) {
+          fx = acc_to_f32(v[j].x);
+          fy = acc_to_f32(v[j].y);
         }
-        if (c0 + 2 * q + 1 < n_cells && acc_nonzero(a[q].y)) {
-          mask |= 1u << (2 * q + 1);
-          v[2 * q + 1] = acc_to_f32(a[q].y);
+        if constexpr (PAIRS) {
+          const int p = warp * kShare + n + __popc(mx & below) + __popc(my & below);
+          const int at = warp * kShare + 64 * j + 2 * lane;
+          if (nx) {
+            s_E[p] = fx;
+            s_at[p] = (uint16_t)at;
+          }
+          if (ny) {
+            s_E[p + (nx ? 1 : 0)] = fy;
+            s_at[p + (nx ? 1 : 0)] = (uint16_t)(at + 1);
+          }
         }
-        if (acc_nonzero(a[q].x) || acc_nonzero(a[q].y)) src[q] = z;  // re-zero what is not zero
+        n += __popc(mx) + __popc(my);
+      }
+      if constexpr (DENSE) {
+        const int c = c0 + 64 * j + 2 * lane;
+        if (j < rows) {
+          if ((A.n_cells & 1) == 0) {  // then c is even and in the row with c + 1
+            if (c < A.n_cells) *reinterpret_cast<float2*>(dense + c) = make_float2(fx, fy);
+          } else {
+            if (c < A.n_cells) dense[c] = fx;
+            if (c + 1 < A.n_cells) dense[c + 1] = fy;
+          }
+        }
       }
     }
-    const int cnt = __popc(mask);
-    int x = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) s_w[warp] = x;
+    if (lane == 0) s_w[warp] = n;
     __syncthreads();
-    int pre = 0, total = 0;
-    for (int w = 0; w < kCThreads / 32; ++w) {
-      if (w < warp) pre += s_w[w];
-      total += s_w[w];
-    }
+    int total = 0;
+#pragma unroll
+    for (int w = 0; w < kCWarps; ++w) total += s_w[w];
     if (warp == 0) {  // publish, look back, publish the prefix
       int64_t excl;
       if (t == 0) {
-        excl = *total_dst;
+        excl = *A.total_dst;
       } else {
         if (lane == 0) atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagAgg | (uint64_t)total);
-        excl = look_back(status, t, flags);
+        excl = look_back(status, t, A.flags);
       }
       if (lane == 0) {
         atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagPrefix | (uint64_t)(excl + total));
         s_base = excl;
-        if (t == n_t - 1) *total_dst = excl + total;
-      }
-    }
-    int lpos = pre + x - cnt;
-#pragma unroll
-    for (int k = 0; k < kCItems; ++k) {
-      if (mask & (1u << k)) {
-        s_id[lpos] = (int32_t)(c0 + k);
-        s_E[lpos] = v[k];
-        ++lpos;
+        if (t % A.cpr == 0 && A.event_offsets_out) A.event_offsets_out[A.ev_lo + row] = excl;
+        if (t == n_t - 1) *A.total_dst = excl + total;
       }
     }
     __syncthreads();
-    const int64_t base = s_base;
-    for (int j = threadIdx.x; j < total; j += kCThreads) {
-      const int64_t pos = base + j;
-      if (pos < capacity) {
-        if (cell_ids) cell_ids[pos] = s_id[j];
-        if (cell_E) cell_E[pos] = s_E[j];
-      }
-    }
-    if (cells_out && c0 < n_cells) {
-      float* dst = cells_out + (int64_t)(ev_lo + row) * n_cells + c0;
-      if (c0 + kCItems <= n_cells && (n_cells & 3) == 0) {
+    if constexpr (PAIRS) {
+      int pre[kCWarps];  // the warps' first pairs in the chunk
+      pre[0] = 0;
 #pragma unroll
-        for (int q = 0; q < kCItems / 4; ++q)
-          reinterpret_cast<float4*>(dst)[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+      for (int w = 1; w < kCWarps; ++w) pre[w] = pre[w - 1] + s_w[w - 1];
+      const int64_t pos = s_base;
+      const int m = (int)max((int64_t)0, min((int64_t)total, A.capacity - pos));
+      if (A.one_run) {
+        // a chunk's pairs as one run (into host memory, over the link: 64
+        // events end to end 1345 us, warp by warp 1370)
+        for (int q = tid; q < m; q += kCThreads) {
+          int first = 0, w = 0;
+#pragma unroll
+          for (int k = 1; k < kCWarps; ++k) {
+            if (q >= pre[k]) {
+              first = pre[k];
+              w = k;
+            }
+          }
+          const int at = w * kShare + q - first;
+          A.cell_ids[pos + q] = cc + s_at[at];
+          A.cell_E[pos + q] = s_E[at];
+        }
       } else {
+        // each warp its own (into device memory: 1024 events 795 us, as one run 846)
+        int first = 0;
 #pragma unroll
-        for (int k = 0; k < kCItems; ++k)
-          if (c0 + k < n_cells) dst[k] = v[k];
+        for (int k = 1; k < kCWarps; ++k) first = warp == k ? pre[k] : first;
+        for (int q = lane; q < n && first + q < m; q += 32) {
+          A.cell_ids[pos + first + q] = cc + s_at[warp * kShare + q];
+          A.cell_E[pos + first + q] = s_E[warp * kShare + q];
+        }
       }
+      __syncthreads();  // the shared arrays are reused
     }
-    if (chunk == 0 && threadIdx.x == 0 && event_offsets_out) event_offsets_out[ev_lo + row] = base;
-    __syncthreads();  // the staging arrays, s_base and s_ticket are reused
   }
   // every CTA has left its loop (and its look-backs) before it counts itself
   // done; the last one resets the state
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     __threadfence();
     s_last = atomicAdd(done, 1ull) == (unsigned long long)gridDim.x - 1;
   }
   __syncthreads();
   if (s_last) {
     __threadfence();
-    for (int64_t i = threadIdx.x; i < n_t; i += kCThreads) status[i] = 0;
-    if (threadIdx.x == 0) {
+    for (int64_t i = tid; i < n_t; i += kCThreads) status[i] = 0;
+    if (tid == 0) {
       *ticket = 0;
       *done = 0;
     }
@@ -169,9 +216,12 @@ cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo
   // persistent CTAs (the ticket order makes every look-back wait end); the
   // offsets continue the call's running output size (per-event mode)
   const int grid = (int)std::min<int64_t>(n_chunks, max_ctas > 0 ? max_ctas : (int64_t)L.num_sms * kCtasPerSm);
-  k_compact_one<<<grid, kCThreads, 0, L.s>>>(w.acc, g.n_cells, g.acc_stride, cpr, n_chunks, ev_lo, tmp.state,
-                                             tmp.cap_tiles, tmp.flags, &w.sizes->nnz_total, cells_out, cell_ids, cell_E,
-                                             event_offsets_out, capacity);
+  const CompactArgs A{w.acc, g.n_cells, g.acc_stride, cpr, ev_lo, max_ctas > 0 ? 1 : 0, n_chunks, tmp.state, tmp.cap_tiles, tmp.flags,
+                      &w.sizes->nnz_total, cells_out, cell_ids, cell_E, event_offsets_out, capacity};
+  if (cells_out && cell_ids) k_compact_one<true, true><<<grid, kCThreads, 0, L.s>>>(A);
+  else if (cells_out) k_compact_one<true, false><<<grid, kCThreads, 0, L.s>>>(A);
+  else if (cell_ids) k_compact_one<false, true><<<grid, kCThreads, 0, L.s>>>(A);
+  else k_compact_one<false, false><<<grid, kCThreads, 0, L.s>>>(A);
   return cudaGetLastError();
 }
 
