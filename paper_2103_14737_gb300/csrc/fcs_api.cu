@@ -1060,16 +1060,17 @@ int fcs_load_params(fcs_params** out, const fcs_geo* geo, const float* frac, con
       (rc = dev_alloc(&d_thr, n_entries * kNBins, &prm->allocs)) ||
       (rc = dev_alloc(&d_guide, n_entries * kGuideCells, &prm->allocs)) ||
       (rc = dev_alloc(&d_lf, kLfactEntries, &prm->allocs)) ||
-      (rc = dev_alloc(&d_lf64, kLfactEntries, &prm->allocs)))
+      (rc = dev_alloc(&d_lf64, kLfactEntries + kRcpEntries, &prm->allocs)))
     return fail(rc);
   // log k! from the host's FP64 lgamma: as is for the FP64 Poisson acceptance
   // test (the value the C definition computes), rounded once for the FP32 test
   std::vector<float> lf(kLfactEntries);
-  std::vector<double> lf64(kLfactEntries);
+  std::vector<double> lf64(kLfactEntries + kRcpEntries);
   for (int k = 0; k < kLfactEntries; ++k) {
     lf64[k] = std::lgamma((double)k + 1.0);
     lf[k] = (float)lf64[k];
   }
+  for (int k = 0; k < kRcpEntries; ++k) lf64[kLfactEntries + k] = 1.0 / (double)(k + 1);
   if ((rc = dev_alloc(&d_w, n_entries * kNBins, &prm->allocs)) || (rc = dev_alloc(&prm->built, n_entries, &prm->allocs)) ||
       (rc = dev_alloc(&prm->list, n_entries + 1, &prm->allocs)) ||
       (rc = dev_alloc(&prm->check, 1, &prm->allocs)))
@@ -1080,7 +1081,7 @@ int fcs_load_params(fcs_params** out, const fcs_geo* geo, const float* frac, con
       (e = cudaMemcpyAsync(d_re, r_edges, (NR + 1) * sizeof(float), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(d_ae, a_edges, (NA + 1) * sizeof(float), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(d_lf, lf.data(), kLfactEntries * sizeof(float), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d_lf64, lf64.data(), kLfactEntries * sizeof(double), cudaMemcpyHostToDevice, s)) !=
+      (e = cudaMemcpyAsync(d_lf64, lf64.data(), lf64.size() * sizeof(double), cudaMemcpyHostToDevice, s)) !=
           cudaSuccess ||
       (e = cudaMemcpyAsync(d_w, shape_w, n_entries * kNBins * sizeof(float), cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = launch_build_tables(d_frac, d_w, (int)n_entries, 1, prm->built, prm->list, prm->list + n_entries, d_thr,

@@ -118,25 +118,33 @@ __device__ __forceinline__ void scales64(const GeoDev& g, int layer, double eta_
   }
 }
 
+// The eta and phi indices in region r.
+__device__ __forceinline__ int32_t eta_index64(const GeoDev& g, int r, double eta) {
+  const int ne = g.n_eta[r];
+  const double te = __ddiv_rn(__dsub_rn(eta, g.eta_lo[r]), g.deta[r]);
+  if (!(te >= 0.0)) return 0;  // also NaN
+  if (te >= (double)ne) return ne - 1;
+  return min((int32_t)floor(te), ne - 1);  // te < n_eta <= 2^22
+}
+__device__ __forceinline__ int32_t phi_index64(const GeoDev& g, int r, double phi) {
+  const int np = g.n_phi[r];
+  double tp = __ddiv_rn(__dsub_rn(phi, g.phi_lo[r]), g.dphi[r]);
+  const double lim = 4503599627370496.0;
+  if (tp > lim) tp = lim;
+  if (!(tp >= -lim)) tp = -lim;  // also NaN
+  const double f = floor(tp);
+  int32_t ip;
+  if (fabs(f) < 2147483648.0) ip = (int32_t)f % np;
+  else ip = (int32_t)((int64_t)f % (int64_t)np);
+  return ip < 0 ? ip + np : ip;
+}
+
 __device__ __forceinline__ int32_t lookup64(const GeoDev& g, int layer, double eta, double phi) {
   const int rb = g.lrb[layer], re = g.lrb[layer + 1];
   int r = rb;
   for (int k = rb + 1; k < re; ++k)
     if (eta >= g.split[k]) r = k;
-  const int ne = g.n_eta[r], np = g.n_phi[r];
-  const double te = __ddiv_rn(__dsub_rn(eta, g.eta_lo[r]), g.deta[r]);
-  int64_t ie;
-  if (!(te >= 0.0)) ie = 0;  // also NaN
-  else if (te >= (double)ne) ie = ne - 1;
-  else ie = (int64_t)floor(te);
-  if (ie > ne - 1) ie = ne - 1;
-  double tp = __ddiv_rn(__dsub_rn(phi, g.phi_lo[r]), g.dphi[r]);
-  const double lim = 4503599627370496.0;
-  if (tp > lim) tp = lim;
-  if (!(tp >= -lim)) tp = -lim;  // also NaN
-  int64_t ip = (int64_t)floor(tp) % (int64_t)np;
-  if (ip < 0) ip += np;
-  return g.cell_off[r] + (int32_t)ie * np + (int32_t)ip;
+  return g.cell_off[r] + eta_index64(g, r, eta) * g.n_phi[r] + phi_index64(g, r, phi);
 }
 
 static __device__ __noinline__ int32_t cell_fp64(const GeoDev& g, const ParamDev& p, int32_t layer,
@@ -741,26 +749,101 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
   }
 }
 
-// FP64 recheck of the queued hits (grid-stride over the queue).
+// FP64 recheck of the queued hits, 32 to a block of two warps (grid-stride over
+// the queue).
+//
+// Bound by latency: a dependent FP64 instruction takes 64 cycles, a division
+// 560, sincos 1750, and a hit's map and lookup are one chain of them, whatever
+// the queue's length.  So the two warps share a hit: the first holds the phi
+// side (sine and cosine, the phi scale and index), the second the eta side (the
+// hyperbolic functions, the eta scale, the region and the eta index), and what
+// one needs of the other goes through shared memory.  cosh and sinh come from
+// one exponential and its reciprocal (within 2 ulp of cosh's value and of
+// sinh's absolute error, both below the rounding of the positions they move),
+// and tanh sinh = sinh^2 / cosh.  Queues of up to some 30,000 hits: 12 to 16 us
+// by one thread a hit and the functions one after the other; 9 to 12 us here (cold).
+struct RecheckShared {
+  double sn[32], cs[32];  // of alpha, by the first warp
+  double sh[32];          // sinh |eta_c|, by the second
+  double s_phi[32];       // |eta_c| > 20: the phi scale, by the second
+  int region[32], ip[32];
+};
+
 template <int MODE>
-__global__ void __launch_bounds__(128) k_recheck(const __grid_constant__ HitKParams kp) {
+__global__ void __launch_bounds__(64) k_recheck(const __grid_constant__ HitKParams kp) {
+  __shared__ RecheckShared sm;
   const WsDev& w = kp.w;
+  const GeoDev& g = kp.g;
   const int64_t n = min(w.sizes->n_recheck, w.recheck_cap);
   const int64_t hit_dbg_base = kp.dbg_hit_cell ? w.sizes->hit_base : 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 q = w.recheck[i];
+  const int lane = threadIdx.x & 31;
+  const bool eta_side = threadIdx.x >= 32;
+  for (int64_t i0 = (int64_t)blockIdx.x * 32; i0 < n; i0 += (int64_t)gridDim.x * 32) {
+    const int64_t i = i0 + lane;
+    const bool have = i < n;
+    const uint2 q = w.recheck[have ? i : i0];
     const TaskRec T = w.tasks[q.x];
     const int32_t layer = T.layer(), event = T.event();
-    const int64_t hb = w.th[q.x];
     const uint4 x = philox4x32_10(
         make_uint4(q.y, (uint32_t)layer | (kPurposeHit << 16), (uint32_t)T.particle, kp.first_event_lo + (uint32_t)event),
         kp.k0, kp.k1);
     const int bin = sample_bin(kp.p, (uint32_t)T.entry() * kNBins, x.x);
-    const int32_t c = cell_fp64(kp.g, kp.p, layer, T.eta_c, T.phi_c, x, bin);
-    deposit_single(kp, event, __fdiv_rn(T.El, (float)w.tn[q.x]), q.x, c, MODE, T.entry(), bin);
-    const int64_t h = hit_dbg_base + hb + q.y;
-    if (kp.dbg_hit_cell && h < kp.dbg_hit_cap) kp.dbg_hit_cell[h] = c;
+    const int ir = bin >> 3, ia = bin & 7;
+    const double r_lo = (double)kp.p.r_edges[ir], r_hi = (double)kp.p.r_edges[ir + 1];
+    const double r = __dadd_rn(r_lo, __dmul_rn(u24d(x.y), __dsub_rn(r_hi, r_lo)));
+    const double R = g.rz[layer];
+    const bool barrel = g.barrel[layer] != 0;
+    const int rb = g.lrb[layer], re = g.lrb[layer + 1];
+    const double ec = (double)T.eta_c, ae = fabs(ec);
+    const bool far = ae > 20.0;  // (sinh^2 overflows at 355; the functions themselves saturate)
+    double sh = 0.0, ch = 0.0, s_eta = 0.0, s_phi = 0.0;
+    if (eta_side) {
+      const double e = exp(ae), ei = __ddiv_rn(1.0, e);
+      ch = __dmul_rn(0.5, __dadd_rn(e, ei));
+      sh = __dmul_rn(0.5, __dsub_rn(e, ei));
+      if (far) scales64(g, layer, ec, &s_eta, &s_phi);
+      sm.sh[lane] = sh;
+      sm.s_phi[lane] = s_phi;
+    } else {
+      const double a_lo = (double)kp.p.a_edges[ia], a_hi = (double)kp.p.a_edges[ia + 1];
+      const double alpha = __dadd_rn(a_lo, __dmul_rn(u24d(x.z), __dsub_rn(a_hi, a_lo)));
+      double sn, cs;
+      sincos(alpha, &sn, &cs);
+      sm.sn[lane] = sn;
+      sm.cs[lane] = cs;
+    }
+    __syncthreads();
+    double pos;  // eta or phi of the hit
+    int rr = rb;
+    if (eta_side) {
+      if (!far) {
+        const double m = __ddiv_rn(barrel ? 1.0 : __dmul_rn(sh, sh), __dmul_rn(R, ch));
+        s_eta = barrel || ec < 0.0 ? m : -m;
+      }
+      pos = __dadd_rn(ec, __dmul_rn(__dmul_rn(r, sm.cs[lane]), s_eta));
+      for (int k = rb + 1; k < re; ++k)
+        if (pos >= g.split[k]) rr = k;
+      sm.region[lane] = rr;
+    } else {
+      s_phi = far ? sm.s_phi[lane] : __ddiv_rn(barrel ? 1.0 : sm.sh[lane], R);
+      pos = __dadd_rn((double)T.phi_c, __dmul_rn(__dmul_rn(r, sm.sn[lane]), s_phi));
+    }
+    __syncthreads();
+    rr = sm.region[lane];
+    int32_t ie = 0;
+    if (eta_side) {
+      ie = eta_index64(g, rr, pos);
+    } else {
+      sm.ip[lane] = phi_index64(g, rr, pos);
+    }
+    __syncthreads();
+    if (eta_side && have) {
+      const int32_t c = g.cell_off[rr] + ie * g.n_phi[rr] + sm.ip[lane];
+      deposit_single(kp, event, __fdiv_rn(T.El, (float)w.tn[q.x]), q.x, c, MODE, T.entry(), bin);
+      const int64_t h = hit_dbg_base + w.th[q.x] + q.y;
+      if (kp.dbg_hit_cell && h < kp.dbg_hit_cap) kp.dbg_hit_cell[h] = c;
+    }
+    // (the next round's first writes are to sn, cs, sh and s_phi, read before the last barrier)
   }
 }
 

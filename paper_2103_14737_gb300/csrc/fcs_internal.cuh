@@ -22,6 +22,7 @@ constexpr int64_t kRecordSlack = 1 << 22;  // slots beyond the hits: the warps' 
 constexpr int kGranule = 128;    // hits per granule of the tile -> task map (divides every tile)
 constexpr int kRecordCountBits = 5;  // deterministic mode: count - 1 in the low 5 bits
 constexpr int kLfactEntries = 8192;  // log k! table for the FP32 Poisson test (k < 8192)
+constexpr int kRcpEntries = 64;      // reciprocals 1 / k behind the FP64 table (k = 1 .. 64)
 
 // Task record: one (event, particle, layer) of the hit loop of Listing 1.
 // 32 bytes (one sector); tasks are stored in (event, particle, layer) order.
@@ -99,7 +100,8 @@ struct ParamDev {
   int32_t n_entries;     // NT * NE * NH * NL
   int32_t n_lfact;       // entries of lfact
   const float* lfact;    // [n_lfact] FP32 of lgamma(k + 1) (host libm, rounded once)
-  const double* lfact64; // [n_lfact] lgamma(k + 1) of the host libm, the FP64 Poisson test's value
+  const double* lfact64; // [n_lfact] lgamma(k + 1) of the host libm, the FP64 Poisson test's value;
+                         // then [kRcpEntries] 1 / k, correctly rounded
   const float* frac;     // [n_entries]
   const float* shape_w;  // [n_entries][128] shape weights (the gradient's likelihood ratios)
   const float* mhe;      // [n_entries]

@@ -273,30 +273,6 @@ __device__ __forceinline__ int32_t ptrs_step_fp32(float mu32, uint32_t layer, ui
   return (int32_t)ptrs_iter32(mu32, c, x);
 }
 
-// A deferred PTRS draw from its uncertain iteration i0 on: iteration i0 in
-// FP64 (the definition), each later one in FP32 where its decisions are
-// certain (they are then the FP64 ones) and in FP64 where they are not.  A
-// warp's time is its longest chain of FP64 iterations, and most draws that
-// reject at i0 are decided in FP32 after it.
-__device__ __noinline__ int64_t ptrs_resume(float mu32, uint32_t layer, uint32_t particle, uint32_t event,
-                                            uint32_t k0, uint32_t k1, const PhiloxRoundKeys& rk,
-                                            const float* lfact, const double* lfact64, int32_t n_lfact, uint32_t i0) {
-  const double mu = (double)mu32;
-  const PtrsConst64 c = ptrs_const64(mu);
-  for (uint32_t i = i0; i < kPtrsMaxIter; ++i) {
-    if (i != i0) {
-      const int32_t k32 = ptrs_step_fp32(mu32, layer, particle, event, rk, lfact, n_lfact, i);
-      if (k32 >= 0) return k32;
-      if (k32 == -1) continue;
-    }
-    double u, V;
-    draw_pair(i, layer, particle, event, k0, k1, &u, &V);
-    const int64_t k = ptrs_iter64(mu, c, u, V, lfact64, n_lfact);
-    if (k >= 0) return k;
-  }
-  return (int64_t)floor(mu);
-}
-
 // Parametrisation entry of a particle (without the layer index).  Energy bin
 // from floor(log2 E): the float's exponent field for normal E, and for a
 // subnormal E = m 2^-149 the position of m's leading bit.  |eta| bin: for an
@@ -648,30 +624,139 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g,
   while (qp.n > 0) ptrs_round(qp, w, rk, first_event_lo, p.lfact, p.n_lfact);
 }
 
-// The deferred draws: the inversion list (front of pdefer) by the FP64
-// definition, then the PTRS list (back of pdefer) resumed at the iteration
-// the FP32 path could not decide; 32 per warp, so that a warp runs one method
-// except at the seam.  A task's mean is recomputed from its record as the
-// build kernel computed it.
-__global__ void __launch_bounds__(128) k_task_poisson64(WsDev w, const float* mhe, PhiloxRoundKeys rk,
-                                                         uint32_t first_event_lo, const float* lfact,
-                                                         const double* lfact64, int32_t n_lfact) {
+// The deferred draws in FP64, the definition's values in the definition's
+// order of operations.
+//
+// Bound by latency: a dependent FP64 instruction takes 64 cycles, a division
+// 560, a square root 680, a logarithm 2090, and a draw is one chain of them,
+// whatever the number of draws.  So the chain is cut:
+//   inversion (front of pdefer, one draw a lane): F_k by four steps a trip, the
+//     division by k from its correctly rounded reciprocal r (a table):
+//     q0 = fl(n r), then q = fl(q0 + fl(n - q0 k) r) with fused operations is
+//     the correctly rounded n / k (Markstein, IBM J. Res. Dev. 34, 1990: r
+//     correctly rounded and q0 within an ulp);
+//   PTRS (back of pdefer, from the iteration the FP32 path could not decide):
+//     four lanes a draw, which share the four divisions and the four
+//     logarithms of an iteration, one each.  Later iterations are taken in
+//     FP32 where their decisions are certain.
+// 1600 draws (64 pile-up events): 25 us by one lane a draw with every function
+// in turn; 13 us here.
+
+// The smallest k with u < F_k (at most kInvMax).
+__device__ __forceinline__ int32_t inversion64(double mu, double u, const double* rcp) {
+  double p = exp(-mu), F = p;
+  int32_t k = 0;
+  while (u >= F && k < kInvMax) {
+    double f[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int32_t kj = k + j + 1;
+      const double n = __dmul_rn(p, mu);
+      if (kj <= kRcpEntries) {
+        const double r = rcp[kj - 1], q0 = __dmul_rn(n, r);
+        p = __fma_rn(__fma_rn(-q0, (double)kj, n), r, q0);
+      } else {
+        p = __ddiv_rn(n, (double)kj);
+      }
+      F = __dadd_rn(F, p);
+      f[j] = F;
+    }
+    // F does not decrease: the steps that u still reaches come first
+    k += u >= f[2] ? 4 : u >= f[1] ? 3 : u >= f[0] ? 2 : 1;
+  }
+  return k;
+}
+
+__global__ void __launch_bounds__(32) k_task_poisson64(WsDev w, const float* mhe, PhiloxRoundKeys rk,
+                                                        uint32_t first_event_lo, const float* lfact,
+                                                        const double* lfact64, int32_t n_lfact) {
+  static_assert(kInvMax % 4 == 0, "four steps a trip end exactly at kInvMax");
+  __shared__ double s_rcp[kRcpEntries];
+  const int lane = threadIdx.x;
   const int64_t n_inv = w.sizes->n_pdefer, n_ptrs = w.sizes->n_pdefer_ptrs;
-  const int64_t n = n_inv + n_ptrs;
-  if (blockIdx.x == 0 && threadIdx.x == 0) w.sizes->n_poisson_fp64 += (uint32_t)n;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (int64_t)gridDim.x * blockDim.x) {
-    const bool inv = q < n_inv;
-    const int32_t t = w.pdefer[inv ? q : w.pdefer_cap - 1 - (q - n_inv)];
-    const TaskRec& r = w.tasks[t];
+  if (blockIdx.x == 0 && lane == 0) w.sizes->n_poisson_fp64 += (uint32_t)(n_inv + n_ptrs);
+  const int64_t inv_items = (n_inv + 31) / 32, items = inv_items + (n_ptrs + 7) / 8;
+  if (blockIdx.x < inv_items) {
+    for (int k = lane; k < kRcpEntries; k += 32) s_rcp[k] = __ldg(lfact64 + n_lfact + k);
+    __syncwarp();
+  }
+  for (int64_t item = blockIdx.x; item < items; item += gridDim.x) {
+    if (item < inv_items) {
+      const int64_t q = item * 32 + lane;
+      if (q < n_inv) {
+        const int32_t t = w.pdefer[q];
+        const TaskRec& r = w.tasks[t];
+        const double mu = (double)__fdiv_rn(r.El, __ldg(mhe + r.entry()));
+        double u, v;
+        draw_pair(0u, (uint32_t)r.layer(), (uint32_t)r.particle, first_event_lo + (uint32_t)r.event(), rk.k[0], rk.k[1],
+                  &u, &v);
+        w.tn[t] = max(inversion64(mu, u, s_rcp), 1);
+      }
+      continue;
+    }
+    const int64_t q = (item - inv_items) * 8 + (lane >> 2);
+    const int j = lane & 3, lead = lane & ~3;
+    const bool have = q < n_ptrs;
+    const int32_t t = w.pdefer[w.pdefer_cap - 1 - (have ? q : (item - inv_items) * 8)];
+    const TaskRec r = w.tasks[t];
     const uint32_t layer = (uint32_t)r.layer(), particle = (uint32_t)r.particle;
     const uint32_t event = first_event_lo + (uint32_t)r.event();
-    const float mu = __fdiv_rn(r.El, __ldg(mhe + r.entry()));
-    int64_t k = inv ? poisson_draw((double)mu, layer, particle, event, rk.k[0], rk.k[1], lfact64, n_lfact, 0u)
-                    : ptrs_resume(mu, layer, particle, event, rk.k[0], rk.k[1], rk, lfact, lfact64, n_lfact,
-                                  (uint32_t)w.tn[t]);
-    if (k < 1) k = 1;
-    if (k > 0x7FFFFFFF) k = 0x7FFFFFFF;
-    w.tn[t] = (int32_t)k;
+    const float mu32 = __fdiv_rn(r.El, __ldg(mhe + r.entry()));
+    const double mu = (double)mu32;
+    uint32_t i = (uint32_t)w.tn[t];
+    __syncwarp();  // every lane has its iteration before one writes the count
+    const double b = __dadd_rn(0.931, __dmul_rn(2.53, __dsqrt_rn(mu)));
+    const double a = __dadd_rn(-0.059, __dmul_rn(0.02483, b));
+    int64_t k = -1;
+    bool open = have, first = true;
+    while (__any_sync(0xffffffffu, open)) {
+      bool need = open;
+      if (open && !first) {
+        const int32_t k32 = ptrs_step_fp32(mu32, layer, particle, event, rk, lfact, n_lfact, i);
+        need = k32 == -2;
+        if (!need) {
+          k = k32;
+          if (k32 == -1) ++i;
+          else open = false;
+        }
+      }
+      first = false;
+      if (__any_sync(0xffffffffu, need)) {
+        // iteration i of the draws that need it (the others' values are not used)
+        double u, V;
+        draw_pair(i, layer, particle, event, rk.k[0], rk.k[1], &u, &V);
+        const double U = __dsub_rn(u, 0.5), us = __dsub_rn(0.5, fabs(U));
+        const double num = j == 0 ? 1.1328 : j == 1 ? 3.6224 : j == 2 ? __dmul_rn(2.0, a) : a;
+        const double den = j == 0 ? __dsub_rn(b, 3.4) : j == 1 ? __dsub_rn(b, 2.0) : j == 2 ? us : __dmul_rn(us, us);
+        const double quo = __ddiv_rn(num, den);  // (us = 0 rejects below)
+        const double invalpha = __dadd_rn(1.1239, __shfl_sync(0xffffffffu, quo, lead));
+        const double vr = __dsub_rn(0.9277, __shfl_sync(0xffffffffu, quo, lead + 1));
+        const double kd = floor(__dadd_rn(
+            __dadd_rn(__dmul_rn(__dadd_rn(__shfl_sync(0xffffffffu, quo, lead + 2), b), U), mu), 0.43));
+        const double hat = __dadd_rn(__shfl_sync(0xffffffffu, quo, lead + 3), b);
+        const double l = log(j == 0 ? V : j == 1 ? invalpha : j == 2 ? hat : mu);
+        const double lV = __shfl_sync(0xffffffffu, l, lead), la = __shfl_sync(0xffffffffu, l, lead + 1);
+        const double lh = __shfl_sync(0xffffffffu, l, lead + 2), lm = __shfl_sync(0xffffffffu, l, lead + 3);
+        if (need) {
+          k = -1;
+          if (us > 0.0) {
+            if (us >= 0.07 && V <= vr) {
+              k = (int64_t)kd;
+            } else if (!(kd < 0.0 || (us < 0.013 && V > us))) {
+              const double lg = (kd < (double)n_lfact) ? __ldg(lfact64 + (int32_t)kd) : lgamma(__dadd_rn(kd, 1.0));
+              if (__dsub_rn(__dadd_rn(lV, la), lh) <= __dsub_rn(__dadd_rn(-mu, __dmul_rn(kd, lm)), lg)) k = (int64_t)kd;
+            }
+          }
+          if (k >= 0) open = false;
+          else ++i;
+        }
+      }
+      if (open && i >= kPtrsMaxIter) {
+        k = (int64_t)floor(mu);
+        open = false;
+      }
+    }
+    if (have && j == 0) w.tn[t] = (int32_t)max((int64_t)1, min(k, (int64_t)0x7FFFFFFF));
   }
 }
 
