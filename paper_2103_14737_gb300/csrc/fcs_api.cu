@@ -350,6 +350,7 @@ constexpr int kRangeThreads = 256;
 __global__ void __launch_bounds__(kRangeThreads) k_range_begin(Sizes* s, const int64_t* __restrict__ off,
                                                                int32_t ev_lo, int32_t ev_hi, int64_t n_particles,
                                                                int64_t pcap) {
+  dependent_start();
   bool bad = false;
   for (int32_t e = ev_lo + (int32_t)threadIdx.x; e < ev_hi; e += kRangeThreads) bad |= off[e + 1] < off[e];
   bad = __syncthreads_or(bad);
@@ -372,6 +373,7 @@ __global__ void __launch_bounds__(kRangeThreads) k_range_begin(Sizes* s, const i
 }
 
 __global__ void k_range_end(Sizes* s) {
+  dependent_start();
   s->task_base += s->n_tasks;
   s->hit_base += s->n_hits;
   s->recheck_total += s->n_recheck;
@@ -379,6 +381,7 @@ __global__ void k_range_end(Sizes* s) {
 
 __global__ void k_call_end(Sizes* s, int64_t* event_offsets_out, int32_t n_events, int64_t capacity,
                            int32_t want_cells) {
+  dependent_start();
   if (event_offsets_out) event_offsets_out[n_events] = s->nnz_total;
   if (want_cells && s->nnz_total > capacity) s->flags |= FCS_FLAG_OUT_CAPACITY;
 }
@@ -467,16 +470,21 @@ int64_t graph_kernel_nodes(cudaGraph_t g) {
 // Poisson counts, hit offsets and tile map, the hit kernel (or one launch per
 // task) and the FP64 recheck.  sync_size: read the hit count back after the
 // scans and grow the hit-dependent buffers.  The range's accumulation rows
-// start at row acc_row0 of the workspace's; *w_out: the view the range used.
+// start at row acc_row0 of the workspace's; dependent: a kernel of this call
+// precedes it on the stream; *w_out: the view the range used.
 int enqueue_range_hits(const CallArgs& a, int32_t ev_lo, int32_t ev_hi, int32_t range, bool sync_size,
-                       const HitCfg& hc, int key_task_bits, int64_t acc_row0, WsDev* w_out) {
+                       const HitCfg& hc, int key_task_bits, int64_t acc_row0, bool dependent, WsDev* w_out) {
   fcs_workspace* ws = a.ws;
   const Launch L{a.s, ws->num_sms};
   const int det = a.cfg.mode == FCS_MODE_DETERMINISTIC;
   cudaEvent_t* tev = a.cfg.timing ? &ws->tev[(size_t)range * 5] : nullptr;
   if (tev) FCS_CUDA(record_stage(tev[0], a.s));
-  k_range_begin<<<1, kRangeThreads, 0, a.s>>>(ws->d_sizes, a.parts.event_offsets, ev_lo, ev_hi, a.n_particles,
-                                              ws->pcap);
+  if (dependent)
+    FCS_CUDA(launch_dependent(k_range_begin, 1, kRangeThreads, 0, a.s, ws->d_sizes, a.parts.event_offsets, ev_lo, ev_hi,
+                              a.n_particles, ws->pcap));
+  else
+    k_range_begin<<<1, kRangeThreads, 0, a.s>>>(ws->d_sizes, a.parts.event_offsets, ev_lo, ev_hi, a.n_particles,
+                                                ws->pcap);
   const uint32_t k0 = (uint32_t)(a.seed & 0xFFFFFFFFu), k1 = (uint32_t)(a.seed >> 32);
   const ScanTmp tmp = ws->scan_tmp();
   auto view = [&]() {
@@ -545,10 +553,10 @@ int enqueue_range(const CallArgs& a, int32_t ev_lo, int32_t ev_hi, int32_t range
                   int key_task_bits) {
   fcs_workspace* ws = a.ws;
   WsDev w{};
-  FCS_TRY(enqueue_range_hits(a, ev_lo, ev_hi, range, sync_size, hc, key_task_bits, 0, &w));
+  FCS_TRY(enqueue_range_hits(a, ev_lo, ev_hi, range, sync_size, hc, key_task_bits, 0, true, &w));
   FCS_TRY(enqueue_range_reduce(a, w, ev_lo, ev_hi - ev_lo, key_task_bits, ws->scan_tmp(), a.s));
   if (a.cfg.timing) FCS_CUDA(record_stage(ws->tev[(size_t)range * 5 + 4], a.s));
-  k_range_end<<<1, 1, 0, a.s>>>(ws->d_sizes);
+  FCS_CUDA(launch_dependent(k_range_end, 1, 1, 0, a.s, ws->d_sizes));
   return FCS_OK;
 }
 
@@ -581,7 +589,8 @@ int enqueue_call(const CallArgs& a, bool sync_size, const HitCfg& hc, int key_ta
   const int32_t W = range_events(a.cfg, a.n_events);
   for (int32_t lo = 0, r = 0; lo < a.n_events; lo += W, ++r)
     FCS_TRY(enqueue_range(a, lo, std::min(a.n_events, lo + W), r, sync_size, hc, key_task_bits));
-  k_call_end<<<1, 1, 0, a.s>>>(ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity, a.cell_ids ? 1 : 0);
+  FCS_CUDA(launch_dependent(k_call_end, 1, 1, 0, a.s, ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity,
+                            a.cell_ids ? 1 : 0));
   FCS_CUDA(cudaGetLastError());
   return FCS_OK;
 }
@@ -678,8 +687,8 @@ int enqueue_waves(const CallArgs& a, const int32_t* type, const float* E, const 
   for (int k = 0; k < nw; ++k) {
     FCS_CUDA(cudaStreamWaitEvent(cs, ws->pev[1 + k], 0));
     WsDev w{};
-    FCS_TRY(enqueue_range_hits(a, bnd[k], bnd[k + 1], k, false, hc, key_task_bits, bnd[k], &w));
-    k_range_end<<<1, 1, 0, cs>>>(ws->d_sizes);
+    FCS_TRY(enqueue_range_hits(a, bnd[k], bnd[k + 1], k, false, hc, key_task_bits, bnd[k], false, &w));
+    FCS_CUDA(launch_dependent(k_range_end, 1, 1, 0, cs, ws->d_sizes));
     FCS_CUDA(cudaEventRecord(ws->pev[1 + nw + k], cs));
     FCS_CUDA(cudaStreamWaitEvent(s_out, ws->pev[1 + nw + k], 0));
     // the compaction runs beside the next wave on a third of the SMs: its
@@ -1556,8 +1565,8 @@ int fcs_simulate_backward(const fcs_geo* geo, const fcs_params* prm, fcs_workspa
   k_call_begin<<<1, 1, 0, s>>>(ws->d_sizes);
   for (int32_t lo = 0; lo < n_events; lo += rows) {
     const int32_t hi = std::min(n_events, lo + rows);
-    k_range_begin<<<1, kRangeThreads, 0, s>>>(ws->d_sizes, particles->event_offsets, lo, hi, n_particles,
-                                              ws->pcap);
+    FCS_CUDA(launch_dependent(k_range_begin, 1, kRangeThreads, 0, s, ws->d_sizes, particles->event_offsets, lo, hi,
+                              n_particles, ws->pcap));
     WsDev w = ws->view();
     FCS_CUDA(launch_task_counts(geo->d, prm->d, *particles, lo, hi, k0, k1, first_event, w, tmp, n_particles,
                                 cfg.energy_interp, L));
@@ -1571,7 +1580,7 @@ int fcs_simulate_backward(const fcs_geo* geo, const fcs_params* prm, fcs_workspa
     const float* g = dL_dcells + (int64_t)lo * geo->d.n_cells;
     FCS_CUDA(launch_hits_grad(geo->d, prm->d, w, lo, k0, k1, first_event, hc, g, ws->grad_acc, ws->grad_touched, L));
     FCS_CUDA(launch_recheck_grad(geo->d, prm->d, w, lo, k0, k1, first_event, g, ws->grad_acc, ws->grad_touched, L));
-    k_range_end<<<1, 1, 0, s>>>(ws->d_sizes);
+    FCS_CUDA(launch_dependent(k_range_end, 1, 1, 0, s, ws->d_sizes));
   }
   FCS_CUDA(launch_grad_finalize(prm->d, ws->grad_acc, ws->grad_touched, d_frac, d_shape_w, L));
   FCS_CUDA(cudaGetLastError());

@@ -63,6 +63,7 @@ struct CompactArgs {
 // DENSE: also the dense rows.  PAIRS: the pairs are wanted (else their number).
 template <bool DENSE, bool PAIRS>
 __global__ void __launch_bounds__(kCThreads, kCtasPerSm) k_compact_one(const CompactArgs A) {
+  dependent_start();
   __shared__ float s_E[PAIRS ? kChunk : 1];
   __shared__ uint16_t s_at[PAIRS ? kChunk : 1];  // place in the chunk
   __shared__ int s_w[kCWarps];
@@ -218,11 +219,15 @@ cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo
   const int grid = (int)std::min<int64_t>(n_chunks, max_ctas > 0 ? max_ctas : (int64_t)L.num_sms * kCtasPerSm);
   const CompactArgs A{w.acc, g.n_cells, g.acc_stride, cpr, ev_lo, max_ctas > 0 ? 1 : 0, n_chunks, tmp.state, tmp.cap_tiles, tmp.flags,
                       &w.sizes->nnz_total, cells_out, cell_ids, cell_E, event_offsets_out, capacity};
-  if (cells_out && cell_ids) k_compact_one<true, true><<<grid, kCThreads, 0, L.s>>>(A);
-  else if (cells_out) k_compact_one<true, false><<<grid, kCThreads, 0, L.s>>>(A);
-  else if (cell_ids) k_compact_one<false, true><<<grid, kCThreads, 0, L.s>>>(A);
-  else k_compact_one<false, false><<<grid, kCThreads, 0, L.s>>>(A);
-  return cudaGetLastError();
+  const auto kernel = cells_out && cell_ids ? k_compact_one<true, true>
+                      : cells_out           ? k_compact_one<true, false>
+                      : cell_ids            ? k_compact_one<false, true>
+                                            : k_compact_one<false, false>;
+  if (max_ctas > 0) {  // on a stream of its own, behind another stream's event
+    kernel<<<grid, kCThreads, 0, L.s>>>(A);
+    return cudaGetLastError();
+  }
+  return launch_dependent(kernel, grid, kCThreads, 0, L.s, A);
 }
 
 int64_t compact_chunks(int32_t n_cells, int32_t rows) {

@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) k_grad_finalize(int32_t n_entries, double
                                                        const float* __restrict__ frac,
                                                        const float* __restrict__ shape_w,
                                                        float* __restrict__ d_frac, float* __restrict__ d_w) {
+  dependent_start();
   const int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (e >= n_entries) return;
@@ -125,9 +126,8 @@ cudaError_t launch_grad_finalize(const ParamDev& p, double* grad_acc, uint8_t* t
                                  float* d_shape_w, const Launch& L) {
   const int64_t threads = (int64_t)p.n_entries * 32;
   if (threads == 0) return cudaSuccess;
-  k_grad_finalize<<<(unsigned)((threads + 255) / 256), 256, 0, L.s>>>(p.n_entries, grad_acc, touched, p.frac,
-                                                                       p.shape_w, d_frac, d_shape_w);
-  return cudaGetLastError();
+  return launch_dependent(k_grad_finalize, (threads + 255) / 256, 256, 0, L.s, p.n_entries, grad_acc, touched, p.frac,
+                          p.shape_w, d_frac, d_shape_w);
 }
 
 cudaError_t launch_check_params(const float* frac, const float* mean_hit_E, const float* shape_w,

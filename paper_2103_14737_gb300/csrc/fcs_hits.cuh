@@ -568,6 +568,7 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
 constexpr int hits_min_ctas(int mode, int block) { return (mode == kModeAtomic ? 9 : 8) * 128 / block; }
 template <int BLOCK, int MODE, bool DBG>
 __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(const __grid_constant__ HitKParams kp) {
+  dependent_start();
   constexpr bool DET = MODE == kModeDet;
   constexpr int NW = BLOCK / 32;
   constexpr int NT = BLOCK > 256 ? 24 : 32;  // staged tasks per warp (static shared memory holds 48 KB)
@@ -771,6 +772,7 @@ struct RecheckShared {
 
 template <int MODE>
 __global__ void __launch_bounds__(64) k_recheck(const __grid_constant__ HitKParams kp) {
+  dependent_start();
   __shared__ RecheckShared sm;
   const WsDev& w = kp.w;
   const GeoDev& g = kp.g;

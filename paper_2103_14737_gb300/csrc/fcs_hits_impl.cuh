@@ -41,8 +41,7 @@ static cudaError_t launch_hits_kernel(const HitKParams& kp, const Launch& L) {
     grid = (kp.h_hi - kp.h_lo + per_cta - 1) / per_cta;
     if (grid <= 0) return cudaSuccess;
   }
-  k_hits<BLOCK, MODE, DBG><<<(unsigned)grid, BLOCK, 0, L.s>>>(kp);
-  return cudaGetLastError();
+  return launch_dependent(k_hits<BLOCK, MODE, DBG>, grid, BLOCK, 0, L.s, kp);
 }
 
 // The validation dumps run in their own instantiation (no gradient-mode dumps).
@@ -72,8 +71,7 @@ cudaError_t launch_hits_t(const HitKParams& kp0, const HitCfg& hc, const Launch&
 template <int MODE>
 cudaError_t launch_recheck_t(const HitKParams& kp, const Launch& L) {
   // FP64 work: small blocks spread the queue over every SM's FP64 pipe
-  k_recheck<MODE><<<L.num_sms * 8, 64, 0, L.s>>>(kp);
-  return cudaGetLastError();
+  return launch_dependent(k_recheck<MODE>, L.num_sms * 8, 64, 0, L.s, kp);
 }
 
 }  // namespace fcs

@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const In* in, Out* out, c
                                                      int64_t* total_dst, int base_from_dst, uint64_t* state,
                                                      int64_t cap_tiles, uint32_t* flags, int32_t* gmap,
                                                      int64_t gmap_cap, int64_t mute_tile) {
+  dependent_start();
   constexpr int TILE = kScanThreads * ITEMS;
   extern __shared__ int64_t s_tile[];  // scan_smem_bytes(ITEMS): element j at j + j / ITEMS
   __shared__ int64_t s_warp[kScanThreads / 32];
@@ -209,11 +210,8 @@ static cudaError_t launch_scan(const In* in, Out* out, const int64_t* n_dev, int
     }
   }
   // the status words are sized for kScanTile-element tiles; larger tiles need fewer
-  k_scan<In, GMAP, ITEMS, Out, ZERO_IN><<<tmp.grid, kScanThreads, smem, s>>>(in, out, n_dev, n_host, total_dst,
-                                                                            base_from_dst ? 1 : 0, tmp.state,
-                                                                            tmp.cap_tiles, tmp.flags, gmap, gmap_cap,
-                                                                            -1);
-  return cudaGetLastError();
+  return launch_dependent(k_scan<In, GMAP, ITEMS, Out, ZERO_IN>, tmp.grid, kScanThreads, smem, s, in, out, n_dev, n_host,
+                          total_dst, base_from_dst ? 1 : 0, tmp.state, tmp.cap_tiles, tmp.flags, gmap, gmap_cap, -1);
 }
 
 cudaError_t launch_scan_i64(const int64_t* in, int64_t* out, const int64_t* n_dev, int64_t n_host,

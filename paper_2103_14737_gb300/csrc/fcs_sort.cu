@@ -47,6 +47,7 @@ constexpr uint32_t kCountMask = (1u << kRecordCountBits) - 1u;
 // offsets: base[r] = poff[first particle of event ev_lo + r].
 __global__ void k_det_bases(const int64_t* __restrict__ event_offsets, int32_t ev_lo, int32_t rows,
                             const int64_t* __restrict__ poff, const Sizes* sz, int64_t* __restrict__ base) {
+  dependent_start();
   const int64_t n_part = sz->n_part, n_tasks = sz->n_tasks;
   const int64_t p0 = event_offsets[ev_lo];
   for (int32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
@@ -64,6 +65,7 @@ __global__ void __launch_bounds__(256) k_det_scatter(const uint64_t* __restrict_
                                                      int cell_shift, uint64_t task_mask, int32_t* __restrict__ cell_off,
                                                      int64_t n_cells_all, uint32_t acc_stride,
                                                      const int64_t* __restrict__ base, uint32_t* __restrict__ out) {
+  dependent_start();
   if (sz->flags & FCS_FLAG_HIT_CAPACITY) return;
   constexpr int R = 4;  // records per thread and trip: their counts-up are in flight together
   const int64_t n = min(sz->n_slots, cap);
@@ -239,6 +241,7 @@ __global__ void __launch_bounds__(256) k_det_fold(const uint32_t* __restrict__ r
                                                   int64_t cap, uint32_t acc_stride, const int64_t* __restrict__ base,
                                                   const float* __restrict__ task_ehit, double* __restrict__ acc,
                                                   int64_t* __restrict__ lists) {
+  dependent_start();
   if (sz->flags & (FCS_FLAG_HIT_CAPACITY | FCS_FLAG_KEY_BITS)) return;
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
@@ -283,6 +286,7 @@ __global__ void __launch_bounds__(256) k_det_fold_mid(const uint32_t* __restrict
                                                       const int64_t* __restrict__ base,
                                                       const float* __restrict__ task_ehit, double* __restrict__ acc,
                                                       const int64_t* __restrict__ lists) {
+  dependent_start();
   static_assert(N == 16 || N == kThreadSortMax, "two mid classes");
   if (sz->flags & (FCS_FLAG_HIT_CAPACITY | FCS_FLAG_KEY_BITS)) return;
   const int64_t n_list = N == 16 ? sz->n_mid : sz->n_mid32;
@@ -306,6 +310,7 @@ __global__ void __launch_bounds__(32 * kBigWarps) k_det_fold_big(uint32_t* __res
                                                                  const float* __restrict__ task_ehit,
                                                                  double* __restrict__ acc,
                                                                  const int64_t* __restrict__ big) {
+  dependent_start();
   __shared__ uint32_t s_rec[kBigWarps][kBigMax];
   __shared__ float s_e[kBigWarps][kBigMax];  // the sorted records' hit energies
   if (sz->flags & (FCS_FLAG_HIT_CAPACITY | FCS_FLAG_KEY_BITS)) return;
@@ -392,26 +397,31 @@ cudaError_t launch_det_reduce(const GeoDev& g, WsDev w, int32_t rows, int key_ta
   int64_t* base = scratch;                                       // [rows] first task of each event
   int32_t* cell_off = reinterpret_cast<int32_t*>(scratch + rows);  // [n_cells_all] segment starts, then ends
   const uint32_t stride = (uint32_t)g.acc_stride;
-  k_det_bases<<<(rows + 255) / 256, 256, 0, L.s>>>(event_offsets, ev_lo, rows, w.poff, w.sizes, base);
-  cudaError_t e = launch_scan_u32_zero(counters, cell_off, n_cells_all, tmp, L.s);
+  cudaError_t e = launch_dependent(k_det_bases, (rows + 255) / 256, 256, 0, L.s, event_offsets, ev_lo, rows, w.poff,
+                                   w.sizes, base);
+  if (e != cudaSuccess) return e;
+  e = launch_scan_u32_zero(counters, cell_off, n_cells_all, tmp, L.s);
   if (e != cudaSuccess) return e;
   const int cell_shift = kRecordCountBits + key_task_bits;
   const uint64_t task_mask = (key_task_bits >= 64) ? ~0ull : ((1ull << key_task_bits) - 1ull);
   uint32_t* segs = reinterpret_cast<uint32_t*>(w.keys_alt);
-  k_det_scatter<<<L.num_sms * 8, 256, 0, L.s>>>(w.keys, w.sizes, w.rec_cap, cell_shift, task_mask, cell_off,
-                                                n_cells_all, stride, base, segs);
+  e = launch_dependent(k_det_scatter, L.num_sms * 8, 256, 0, L.s, w.keys, w.sizes, w.rec_cap, cell_shift, task_mask,
+                       cell_off, n_cells_all, stride, base, segs);
+  if (e != cudaSuccess) return e;
   // the slot array is free after the scatter: it lists the segments of more
   // than 8 records
   int64_t* lists = reinterpret_cast<int64_t*>(w.keys);
-  k_det_fold<<<L.num_sms * fold_resident_blocks(), 256, 0, L.s>>>(segs, cell_off, n_cells_all, w.sizes, w.rec_cap,
-                                                                  stride, base, w.tehit, w.acc, lists);
-  k_det_fold_mid<16><<<L.num_sms * 4, 256, 0, L.s>>>(segs, cell_off, n_cells_all, w.sizes, w.rec_cap, stride, base,
-                                                     w.tehit, w.acc, lists);
-  k_det_fold_mid<kThreadSortMax><<<L.num_sms * 2, 256, 0, L.s>>>(segs, cell_off, n_cells_all, w.sizes, w.rec_cap,
-                                                                stride, base, w.tehit, w.acc, lists);
-  k_det_fold_big<<<L.num_sms * 4, 32 * kBigWarps, 0, L.s>>>(segs, cell_off, n_cells_all, w.sizes, w.rec_cap, stride,
-                                                            base, w.tehit, w.acc, lists);
-  return cudaGetLastError();
+  e = launch_dependent(k_det_fold, L.num_sms * fold_resident_blocks(), 256, 0, L.s, segs, cell_off, n_cells_all, w.sizes,
+                       w.rec_cap, stride, base, w.tehit, w.acc, lists);
+  if (e != cudaSuccess) return e;
+  e = launch_dependent(k_det_fold_mid<16>, L.num_sms * 4, 256, 0, L.s, segs, cell_off, n_cells_all, w.sizes, w.rec_cap,
+                       stride, base, w.tehit, w.acc, lists);
+  if (e != cudaSuccess) return e;
+  e = launch_dependent(k_det_fold_mid<kThreadSortMax>, L.num_sms * 2, 256, 0, L.s, segs, cell_off, n_cells_all, w.sizes,
+                       w.rec_cap, stride, base, w.tehit, w.acc, lists);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(k_det_fold_big, L.num_sms * 4, 32 * kBigWarps, 0, L.s, segs, cell_off, n_cells_all, w.sizes,
+                          w.rec_cap, stride, base, w.tehit, w.acc, lists);
 }
 
 }  // namespace fcs

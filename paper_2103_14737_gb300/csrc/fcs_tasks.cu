@@ -368,6 +368,7 @@ __device__ __forceinline__ int32_t interp_entry(const ParamDev& p, int32_t entry
 __global__ void __launch_bounds__(128) k_particle_count(const ParamDev p, const fcs_particles parts, int32_t ev_lo,
                                                         int32_t ev_hi, WsDev w, int energy_interp, uint32_t k0,
                                                         uint32_t k1, uint32_t first_event_lo) {
+  dependent_start();
   const int64_t pb = parts.event_offsets[ev_lo];
   const int64_t P = w.sizes->n_part;  // checked against the capacity and n_particles
   for (int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; li < P;
@@ -523,6 +524,7 @@ __device__ __forceinline__ uint32_t home_region(const GeoDev& g, int l, float et
 __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g, const ParamDev p,
                                                                  const fcs_particles parts, int32_t ev_lo, WsDev w,
                                                                  PhiloxRoundKeys rk, uint32_t first_event_lo) {
+  dependent_start();
   __shared__ DrawEnt s_e[2][kBuildWarps][kDrawQ];  // inversion and PTRS queues
   __shared__ uint8_t s_it[2][kBuildWarps][kDrawQ];
   __shared__ float s_rcp[kInvMax + 1];  // 1 / k, correctly rounded
@@ -670,6 +672,7 @@ __device__ __forceinline__ int32_t inversion64(double mu, double u, const double
 __global__ void __launch_bounds__(32) k_task_poisson64(WsDev w, const float* mhe, PhiloxRoundKeys rk,
                                                         uint32_t first_event_lo, const float* lfact,
                                                         const double* lfact64, int32_t n_lfact) {
+  dependent_start();
   static_assert(kInvMax % 4 == 0, "four steps a trip end exactly at kInvMax");
   __shared__ double s_rcp[kRcpEntries];
   const int lane = threadIdx.x;
@@ -801,6 +804,7 @@ __global__ void __launch_bounds__(128) k_poisson_audit(const float* mu, int64_t 
 // holding its first hit) again when the call grew it after the scan that
 // wrote it (fill_map).
 __global__ void k_task_finish(WsDev w, fcs_debug dbg, int has_dbg, int fill_map) {
+  dependent_start();
   const int64_t T = min(w.sizes->n_tasks, w.task_cap);
   const int64_t H = w.sizes->n_hits;
   const bool map_ok = fill_map && H <= w.gmap_cap * (int64_t)kGranule;
@@ -854,8 +858,10 @@ cudaError_t launch_task_counts(const GeoDev& g, const ParamDev& p, const fcs_par
   // one thread per particle / task where the grid allows (these kernels wait
   // on dependent loads: more threads in flight, not fewer, hide them)
   const int gp = grid_for(n_part_max, L);
-  k_particle_count<<<gp, 128, 0, L.s>>>(p, parts, ev_lo, ev_hi, w, energy_interp, k0, k1, (uint32_t)first_event);
-  cudaError_t e = launch_scan_i64(w.pcount, w.poff, &w.sizes->n_part, 0, &w.sizes->n_tasks, 0, tmp, L.s);
+  cudaError_t e = launch_dependent(k_particle_count, gp, 128, 0, L.s, p, parts, ev_lo, ev_hi, w, energy_interp, k0, k1,
+                                   (uint32_t)first_event);
+  if (e != cudaSuccess) return e;
+  e = launch_scan_i64(w.pcount, w.poff, &w.sizes->n_part, 0, &w.sizes->n_tasks, 0, tmp, L.s);
   if (e != cudaSuccess) return e;
   // the build kernel loops grid-stride: one wave of resident blocks
   static std::atomic<int> occ_by_device[kMaxDevices];
@@ -869,11 +875,13 @@ cudaError_t launch_task_counts(const GeoDev& g, const ParamDev& p, const fcs_par
   const PhiloxRoundKeys rk = philox_round_keys(k0, k1);
   const int gb = (int)std::min<int64_t>((std::max<int64_t>(n_part_max, 1) + 32 * kBuildWarps - 1) / (32 * kBuildWarps),
                                         (int64_t)L.num_sms * occ);
-  k_task_build<<<gb, 32 * kBuildWarps, 0, L.s>>>(g, p, parts, ev_lo, w, rk, (uint32_t)first_event);
+  e = launch_dependent(k_task_build, gb, 32 * kBuildWarps, 0, L.s, g, p, parts, ev_lo, w, rk, (uint32_t)first_event);
+  if (e != cudaSuccess) return e;
   // the FP64 pipe is narrow: one warp per block spreads the few deferred draws
   // over every SM
-  k_task_poisson64<<<L.num_sms * 8, 32, 0, L.s>>>(w, p.mhe, rk, (uint32_t)first_event, p.lfact, p.lfact64,
-                                                   p.n_lfact);
+  e = launch_dependent(k_task_poisson64, L.num_sms * 8, 32, 0, L.s, w, p.mhe, rk, (uint32_t)first_event, p.lfact,
+                       p.lfact64, p.n_lfact);
+  if (e != cudaSuccess) return e;
   // the scan counts the tasks actually written (n_tasks <= task_cap by construction)
   return launch_scan_hits(w.tn, w.th, &w.sizes->n_tasks, &w.sizes->n_hits, w.gmap, w.gmap_cap, tmp, L.s);
 }
@@ -882,8 +890,7 @@ cudaError_t launch_task_finish(WsDev w, const fcs_debug* dbg, int fill_map, int6
   if (!dbg && !fill_map) return cudaSuccess;  // the scan wrote the tile map
   fcs_debug d{};
   if (dbg) d = *dbg;
-  k_task_finish<<<grid_for(n_task_max, L), 128, 0, L.s>>>(w, d, dbg ? 1 : 0, fill_map);
-  return cudaGetLastError();
+  return launch_dependent(k_task_finish, grid_for(n_task_max, L), 128, 0, L.s, w, d, dbg ? 1 : 0, fill_map);
 }
 
 cudaError_t launch_poisson_audit(const ParamDev& p, const float* mu, int64_t n, uint32_t k0, uint32_t k1,
