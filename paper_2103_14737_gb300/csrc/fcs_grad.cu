@@ -12,8 +12,8 @@
 //   dL/dw[e][b] = A[e][b] / w_b - sum_j A[e][j] / W     (A / w := 0 where w_b = 0)
 // The hit kernel in gradient mode regenerates every hit (Philox, bin, cell,
 // FP64 recheck of uncertain cells) exactly as the forward pass does, gathers
-// dL/dE_cell, sums E_hit dL/dE_cell per (entry, bin) over each warp's hits
-// and adds the sums to A in FP64; the finalize kernel turns A into the two
+// dL/dE_cell and adds each E_hit dL/dE_cell to its (entry, bin) of A in FP64;
+// the finalize kernel turns A into the two
 // gradients for the entries that received hits and clears A for the next call.
 #include "fcs_hits_impl.cuh"
 

@@ -367,8 +367,8 @@ __device__ __forceinline__ FastHit fast_cell(const HitSmemTables& tb, const Tile
 }
 
 // ---- warp-level deposit / record emission -----------------------------------
-// Deterministic mode: the first lane of each group of equal (cell, task) keys
-// in the warp writes the group's record (count - 1 in the low bits) and counts
+// Deterministic mode: the first lane of each group (peers: its lanes) of equal
+// (cell, task) keys in the warp writes the group's record (count - 1 in the low bits) and counts
 // it in the cell's uint32 counter (the accumulation row).  A warp writes its
 // records contiguously into chunks of kRecordChunk slots that it takes from
 // the range's slot counter (a round that does not fit continues in the next
@@ -382,12 +382,9 @@ struct RecordChunk {
   int fill = kRecordChunk;  // no chunk yet
 };
 
-__device__ __forceinline__ unsigned emit_records(bool ok, unsigned long long gkey, uint32_t cell, RecordChunk& ch,
-                                                 const WsDev& w) {
+__device__ __forceinline__ unsigned emit_records(bool ok, unsigned peers, unsigned long long gkey, uint32_t cell,
+                                                 RecordChunk& ch, const WsDev& w) {
   const int lane = threadIdx.x & 31;
-  const unsigned m = __ballot_sync(0xffffffffu, ok);
-  unsigned peers = 0;
-  if (ok) peers = __match_any_sync(m, gkey);
   const bool lead = ok && (lane == __ffs(peers) - 1);
   const unsigned lm = __ballot_sync(0xffffffffu, lead);
   const int cnt = __popc(lm);
@@ -423,24 +420,12 @@ __device__ __forceinline__ void close_records(const RecordChunk& ch, const WsDev
     if (ch.base + j < w.rec_cap) w.keys[ch.base + j] = ~0ull;
 }
 
-// Sum of v over each group of lanes with equal keys, added by the group's
-// first lane to grad_acc[key] in FP64 (key = entry * 128 + bin).  s_v: this
-// warp's 32 floats of shared memory; groups sum in ascending lane order.
-__device__ __forceinline__ void grad_warp(bool ok, uint32_t key, float v, float* s_v, const HitKParams& kp) {
-  const int lane = threadIdx.x & 31;
-  const unsigned m = __ballot_sync(0xffffffffu, ok);
-  s_v[lane] = v;
-  __syncwarp();
-  if (ok) {
-    const unsigned peers = __match_any_sync(m, key);
-    if (lane == __ffs(peers) - 1) {
-      float sum = 0.0f;
-      for (unsigned q = peers; q; q &= q - 1) sum += s_v[__ffs(q) - 1];
-      atomicAdd(kp.grad_acc + key, (double)sum);
-      kp.grad_touched[key >> 7] = 1;
-    }
-  }
-  __syncwarp();
+// A hit's E_hit dL/dE_cell, added in FP64 to the score of its (entry, bin).
+// Each hit adds by itself: the 32 hits of a step fall into some 25 (entry, bin)
+// pairs, so matching them first (2.2 cycles of the SM per distinct key) cost
+// more than it saved (64 events, the whole backward call: 1348 to 1003 us).
+__device__ __forceinline__ void grad_add(const HitKParams& kp, uint32_t key, float v) {
+  atomicAdd(kp.grad_acc + key, (double)v);
 }
 
 __device__ __forceinline__ void deposit_single(const HitKParams& kp, int32_t event, float Ehit, int64_t task_rel,
@@ -474,7 +459,7 @@ __device__ __forceinline__ void deposit_single(const HitKParams& kp, int32_t eve
 // here in FP64, as the recheck kernel would.  Called by the whole warp; out of
 // line, as it runs once in some 50 warp steps (2 % of the hits, 32 at a time).
 template <int MODE, bool DBG>
-static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool have, uint2 th, float* s_v) {
+static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool have, uint2 th) {
   const WsDev& w = kp.w;
   TaskRec T{};
   uint4 x = make_uint4(0u, 0u, 0u, 0u);
@@ -509,8 +494,9 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
   const int64_t row = T.event() - kp.ev_lo;
   const float Ehit = ok ? __fdiv_rn(T.El, (float)w.tn[th.x]) : 0.0f;
   if constexpr (MODE == kModeGrad) {
-    const float v = ok ? __fmul_rn(Ehit, __ldg(kp.grad_in + row * kp.g.n_cells + c)) : 0.0f;
-    grad_warp(ok, ((uint32_t)T.entry() << 7) | (uint32_t)bin, v, s_v, kp);
+    if (ok)
+      grad_add(kp, ((uint32_t)T.entry() << 7) | (uint32_t)bin,
+               __fmul_rn(Ehit, __ldg(kp.grad_in + row * kp.g.n_cells + c)));
   } else if constexpr (MODE == kModeAtomic) {
     if (ok) acc_add(w.acc + row * kp.g.acc_stride + c, Ehit);
   } else {
@@ -562,12 +548,12 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
 // (Finishing the searches in the loop with two more loads: 610.  Without any
 // put-off hit, wrongly, it would be 500.)
 //
-// MIN CTAs per SM: the modes' best of 7 to 10.  DBG: the validation dumps of
+// 9 CTAs of 128 threads per SM in every mode (of 7 to 10 tried).  DBG: the validation dumps of
 // fcs_debug (a separate instantiation, so that the production kernel carries
 // none of their code).
-constexpr int hits_min_ctas(int mode, int block) { return (mode == kModeAtomic ? 9 : 8) * 128 / block; }
+constexpr int hits_min_ctas(int block) { return 9 * 128 / block; }
 template <int BLOCK, int MODE, bool DBG>
-__global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(const __grid_constant__ HitKParams kp) {
+__global__ void __launch_bounds__(BLOCK, hits_min_ctas(BLOCK)) k_hits(const __grid_constant__ HitKParams kp) {
   dependent_start();
   constexpr bool DET = MODE == kModeDet;
   constexpr int NW = BLOCK / 32;
@@ -579,7 +565,6 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
   __shared__ __align__(16) TileTask s_task[NW][NT];
   __shared__ uint32_t s_start[NW][32];  // bit i of the pass: a task other than its first starts at hit i
   __shared__ uint2 s_def[NW][96];       // hits put off (task, hit), fewer than 32 between rounds of two steps
-  __shared__ float s_gv[MODE == kModeGrad ? BLOCK : 1];  // gradient mode
   __shared__ unsigned long long s_recs;  // deterministic mode: records of this CTA
   load_tables(tb, kp.p);
   if (DET && threadIdx.x == 0) s_recs = 0;
@@ -607,7 +592,6 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
   unsigned long long recs = 0;  // deterministic mode: this warp's records
   RecordChunk chunk;            //   and the slots it writes them to
   int n_def = 0;                // this warp's hits in s_def
-  float* const s_v = MODE == kModeGrad ? s_gv + warp * 32 : nullptr;
   // The first two thirds of the tickets go to the warps in turn, the rest
   // through the queue (its counter serves a ticket in 2.2 ns), which evens out
   // the warps' speeds; calls of many tickets a warp take all from the queue,
@@ -648,6 +632,7 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
           if constexpr (DET) {
             if (t.rel >= 0) w.tehit[t0 + lane] = t.Ehit;
           }
+          if constexpr (MODE == kModeGrad) kp.grad_touched[t.gbase / kNBins] = 1;  // the task has hits
         }
       }
       end = __shfl_sync(kAll, after, NT - 1);
@@ -684,21 +669,22 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
         const bool ok = valid && f.sure && !gb.search;
         if constexpr (MODE == kModeGrad) {
           // dL/dE_cell of the hit's cell times its energy, summed per (entry, bin)
-          const float v = ok ? __fmul_rn(T.Ehit, __ldg(kp.grad_in + f.cell)) : 0.0f;
-          grad_warp(ok, T.gbase | (uint32_t)bin, v, s_v, kp);
-        } else if constexpr (!DET) {
+          if (ok) grad_add(kp, T.gbase | (uint32_t)bin, __fmul_rn(T.Ehit, __ldg(kp.grad_in + f.cell)));
+        } else {
           // the low 27 bits of the row offset + cell tell a task's cells apart
           // (n_cells < 2^27): with the task in the pass they identify (address, hit energy)
           const unsigned m = __ballot_sync(kAll, ok);
           const unsigned peers =
               m & (kp.key32 ? __match_any_sync(kAll, (f.cell << 5) | (uint32_t)d.tl)
                             : __match_any_sync(kAll, ((unsigned long long)(uint32_t)d.tl << 32) | f.cell));
-          if (ok && (peers & lanes_below) == 0u)  // the group's first lane deposits
-            acc_add(w.acc + f.cell, __fmul_rn((float)__popc(peers), T.Ehit));
-        } else {
-          const unsigned long long gkey =
-              ((unsigned long long)f.cell << kp.key_task_bits) | (unsigned long long)(t0 + d.tl);
-          recs += emit_records(ok, gkey, f.cell, chunk, w);
+          if constexpr (!DET) {
+            if (ok && (peers & lanes_below) == 0u)  // the group's first lane deposits
+              acc_add(w.acc + f.cell, __fmul_rn((float)__popc(peers), T.Ehit));
+          } else {
+            const unsigned long long gkey =
+                ((unsigned long long)f.cell << kp.key_task_bits) | (unsigned long long)(t0 + d.tl);
+            recs += emit_records(ok, peers, gkey, f.cell, chunk, w);
+          }
         }
         if constexpr (DBG) {
           const int64_t h = w.sizes->hit_base + h0 + k * 32 + lane;
@@ -730,7 +716,7 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
           __syncwarp();
           do {
             n_def -= 32;
-            deferred_hits<MODE, DBG>(kp, true, s_def[warp][n_def + lane], s_v);
+            deferred_hits<MODE, DBG>(kp, true, s_def[warp][n_def + lane]);
           } while (n_def >= 32);
           __syncwarp();
         }
@@ -741,7 +727,7 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(MODE, BLOCK)) k_hits(cons
     tile = __shfl_sync(kAll, next, 0);
   }
   __syncwarp();
-  if (n_def) deferred_hits<MODE, DBG>(kp, lane < n_def, s_def[warp][lane], s_v);
+  if (n_def) deferred_hits<MODE, DBG>(kp, lane < n_def, s_def[warp][lane]);
   if constexpr (DET) {
     close_records(chunk, w);
     if (lane == 0 && recs) atomicAdd(&s_recs, recs);
