@@ -72,7 +72,8 @@ __global__ void __launch_bounds__(256) k_table_list(const float* __restrict__ fr
 // ten times that; the FP64 pipe takes one warp instruction in 16 cycles).
 // 122,400 entries, 28 % of them with a fraction, in a training step's update:
 // 0.64 ms for one thread per entry reading its own row and dividing, 0.75 ms
-// with the 256-cell guide, 0.04 ms here.
+// with the 256-cell guide, 0.07 ms here (0.095 before the rows were loaded four at
+// a time and the sweep kept the next thresholds in registers).
 constexpr int kTableWarps = 2;
 constexpr int kTableRow = 33;  // [bin][lane], padded for the row-wise accesses
 
@@ -91,11 +92,20 @@ __global__ void __launch_bounds__(32 * kTableWarps) k_build_tables(const float* 
     const int cnt = min(32, n - g);
     const int mine = list[g + min(lane, cnt - 1)];
     __syncwarp();
-    for (int j = 0; j < cnt; ++j) {
-      const int e = __shfl_sync(0xffffffffu, mine, j);
+    // (rows past cnt are the last entry's again; four rows' loads in flight)
+#pragma unroll 1
+    for (int j0 = 0; j0 < 32; j0 += 4) {
+      float v[4][4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        rows[(lane + 32 * q) * kTableRow + j] = __float_as_uint(__ldg(shape_w + (int64_t)e * kNBins + lane + 32 * q));
+      for (int j = 0; j < 4; ++j) {
+        const int e = __shfl_sync(0xffffffffu, mine, j0 + j);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) v[j][q] = __ldg(shape_w + (int64_t)e * kNBins + lane + 32 * q);
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rows[(lane + 32 * q) * kTableRow + j0 + j] = __float_as_uint(v[j][q]);
     }
     __syncwarp();
     double C = 0.0;
@@ -133,6 +143,7 @@ __global__ void __launch_bounds__(32 * kTableWarps) k_build_tables(const float* 
       rows[k * kTableRow + lane] = T;
     }
     __syncwarp();
+#pragma unroll 4
     for (int j = 0; j < cnt; ++j) {
       const int e = __shfl_sync(0xffffffffu, mine, j);
 #pragma unroll
@@ -140,24 +151,35 @@ __global__ void __launch_bounds__(32 * kTableWarps) k_build_tables(const float* 
     }
     // lo_j = first k < K with (j << 24) < T[k], else K (monotone sweep); cell j
     // ends where the next begins, the last one at K
+    // (Tk: the threshold k, and Tn the one after it, loaded ahead of its use)
     int k = 0;
-    while (k < K && rows[k * kTableRow + lane] == 0u) ++k;  // lo_0: bins of zero weight before the first
+    uint32_t Tk = rows[lane], Tn = rows[kTableRow + lane];
+    auto step = [&]() {
+      ++k;
+      Tk = Tn;
+      Tn = rows[min(k + 1, kNBins - 1) * kTableRow + lane];
+    };
+    while (k < K && Tk == 0u) step();  // lo_0: bins of zero weight before the first
     for (int j0 = 0; j0 < kGuideCells; j0 += 32) {
+#pragma unroll 4
       for (int j = 0; j < 32; ++j) {
         const int lo = k;
-        const uint64_t top = (uint64_t)(j0 + j + 1) << 24;
-        const uint32_t t0 = lo < K ? rows[lo * kTableRow + lane] : 0u;
+        const uint32_t base = (uint32_t)(j0 + j) << 24;
+        const uint32_t t0 = Tk;
+        int span = 0;
         if (j0 + j + 1 < kGuideCells) {
-          while (k < K && top >= rows[k * kTableRow + lane]) ++k;
+          while (k < K && base + 0x1000000u >= Tk) {
+            step();
+            ++span;
+          }
         } else {
-          k = max(K, 0);
+          span = max(K, 0) - k;
         }
-        const int span = k - lo;
-        cells[j * kTableRow + lane] =
-            good ? guide_cell(span >= 1 ? t0 - ((uint32_t)(j0 + j) << 24) - 1u : kGuideNever, lo, span)
-                 : guide_cell(kGuideNever, 0, 0);
+        cells[j * kTableRow + lane] = guide_cell(good && span >= 1 ? t0 - base - 1u : kGuideNever, good ? lo : 0,
+                                                 good ? span : 0);
       }
       __syncwarp();
+#pragma unroll 8
       for (int j = 0; j < cnt; ++j) {
         const int e = __shfl_sync(0xffffffffu, mine, j);
         guide[(int64_t)e * kGuideCells + j0 + lane] = cells[lane * kTableRow + j];
