@@ -379,11 +379,17 @@ __global__ void k_range_end(Sizes* s) {
   s->recheck_total += s->n_recheck;
 }
 
+// host: the workspace's pinned copy (mapped), written here so that a
+// synchronous call needs no copy behind its kernels (one electron: 4 us).
 __global__ void k_call_end(Sizes* s, int64_t* event_offsets_out, int32_t n_events, int64_t capacity,
-                           int32_t want_cells) {
+                           int32_t want_cells, Sizes* host) {
   dependent_start();
   if (event_offsets_out) event_offsets_out[n_events] = s->nnz_total;
   if (want_cells && s->nnz_total > capacity) s->flags |= FCS_FLAG_OUT_CAPACITY;
+  if (host) {
+    *host = *s;
+    __threadfence_system();
+  }
 }
 
 __global__ void k_empty_offsets(int64_t* event_offsets_out, int32_t n_events) {
@@ -590,7 +596,7 @@ int enqueue_call(const CallArgs& a, bool sync_size, const HitCfg& hc, int key_ta
   for (int32_t lo = 0, r = 0; lo < a.n_events; lo += W, ++r)
     FCS_TRY(enqueue_range(a, lo, std::min(a.n_events, lo + W), r, sync_size, hc, key_task_bits));
   FCS_CUDA(launch_dependent(k_call_end, 1, 1, 0, a.s, ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity,
-                            a.cell_ids ? 1 : 0));
+                            a.cell_ids ? 1 : 0, ws->h_sizes));
   FCS_CUDA(cudaGetLastError());
   return FCS_OK;
 }
@@ -697,7 +703,8 @@ int enqueue_waves(const CallArgs& a, const int32_t* type, const float* E, const 
     // small calls; half slowed the next wave on large ones)
     FCS_TRY(enqueue_range_reduce(a, w, bnd[k], bnd[k + 1] - bnd[k], key_task_bits, tmp2, s_out, ws->num_sms / 3));
   }
-  k_call_end<<<1, 1, 0, s_out>>>(ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity, a.cell_ids ? 1 : 0);
+  k_call_end<<<1, 1, 0, s_out>>>(ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity, a.cell_ids ? 1 : 0,
+                                  ws->h_sizes);
   FCS_CUDA(cudaEventRecord(ws->pev[1 + 2 * nw], s_out));
   FCS_CUDA(cudaStreamWaitEvent(cs, ws->pev[1 + 2 * nw], 0));
   FCS_CUDA(cudaGetLastError());
@@ -1347,14 +1354,12 @@ int fcs_simulate_events(const fcs_geo* geo, const fcs_params* prm, fcs_workspace
   const bool size_mid_call = cfg.sync != 0 && cfg.batched == 1 && ws->gmap_cap == 0;
   FCS_TRY(enqueue_call(a, size_mid_call, hc, key_task_bits));
   if (!cfg.sync) return ok();
-  FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
-  FCS_CUDA(cudaStreamSynchronize(s));
+  FCS_CUDA(cudaStreamSynchronize(s));  // (k_call_end has written h_sizes)
   if (ws->h_sizes->flags & FCS_FLAG_HIT_CAPACITY) {
     // the call outgrew the workspace: size it for the whole call's hits (they
     // bound every event range's) and run again
     FCS_TRY(ws_reserve_hits(ws, ws->h_sizes->hit_base, cfg.mode));
     FCS_TRY(enqueue_call(a, false, hc, key_task_bits));
-    FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
     FCS_CUDA(cudaStreamSynchronize(s));
   }
   return status_from(*ws->h_sizes, stats);
@@ -1471,8 +1476,7 @@ int fcs_simulate_events_host(const fcs_geo* geo, const fcs_params* prm, fcs_work
       return ok();
     }
     if (rc2 == FCS_OK) {
-      FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
-      FCS_CUDA(cudaStreamSynchronize(s));
+      FCS_CUDA(cudaStreamSynchronize(s));  // (k_call_end has written h_sizes)
       if (!(ws->h_sizes->flags & FCS_FLAG_HIT_CAPACITY)) return status_from(*ws->h_sizes, stats);
       FCS_TRY(ws_reserve_hits(ws, ws->h_sizes->hit_base, cfg.mode));
     } else if (rc2 != FCS_E_UNSUPPORTED) {
@@ -1494,8 +1498,7 @@ int fcs_simulate_events_host(const fcs_geo* geo, const fcs_params* prm, fcs_work
       gcfg.timing = 0;
       FCS_TRY(fcs_simulate_events(geo, prm, ws, &parts, n_particles, n_events, seed, first_event, &gcfg, nullptr,
                                   m_ids, m_cE, m_oout, capacity, nullptr, nullptr, s));
-      FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
-      FCS_CUDA(cudaStreamSynchronize(s));
+      FCS_CUDA(cudaStreamSynchronize(s));  // (k_call_end has written h_sizes)
       if (!(ws->h_sizes->flags & FCS_FLAG_HIT_CAPACITY)) return status_from(*ws->h_sizes, stats);
       FCS_TRY(ws_reserve_hits(ws, ws->h_sizes->hit_base, cfg.mode));
     }
@@ -1561,33 +1564,41 @@ int fcs_simulate_backward(const fcs_geo* geo, const fcs_params* prm, fcs_workspa
   const Launch L{s, ws->num_sms};
   const uint32_t k0 = (uint32_t)(seed & 0xFFFFFFFFu), k1 = (uint32_t)(seed >> 32);
   const ScanTmp tmp = ws->scan_tmp();
-  ws->grad_dirty = true;
-  k_call_begin<<<1, 1, 0, s>>>(ws->d_sizes);
-  for (int32_t lo = 0; lo < n_events; lo += rows) {
-    const int32_t hi = std::min(n_events, lo + rows);
-    FCS_CUDA(launch_dependent(k_range_begin, 1, kRangeThreads, 0, s, ws->d_sizes, particles->event_offsets, lo, hi,
-                              n_particles, ws->pcap));
-    WsDev w = ws->view();
-    FCS_CUDA(launch_task_counts(geo->d, prm->d, *particles, lo, hi, k0, k1, first_event, w, tmp, n_particles,
-                                cfg.energy_interp, L));
-    if (cfg.sync) {
-      FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
-      FCS_CUDA(cudaStreamSynchronize(s));
-      FCS_TRY(ws_reserve_hits(ws, ws->h_sizes->n_hits, FCS_MODE_ATOMIC));
-      w = ws->view();
+  // A sync call of one range whose workspace has been sized runs without the
+  // mid-call read of the hit count; if it outgrows the workspace its hit kernel
+  // adds nothing, so the call is run again with the workspace grown.
+  bool size_mid_call = cfg.sync != 0 && (rows < n_events || ws->gmap_cap == 0);
+  for (int attempt = 0;; ++attempt) {
+    ws->grad_dirty = true;
+    k_call_begin<<<1, 1, 0, s>>>(ws->d_sizes);
+    for (int32_t lo = 0; lo < n_events; lo += rows) {
+      const int32_t hi = std::min(n_events, lo + rows);
+      FCS_CUDA(launch_dependent(k_range_begin, 1, kRangeThreads, 0, s, ws->d_sizes, particles->event_offsets, lo, hi,
+                                n_particles, ws->pcap));
+      WsDev w = ws->view();
+      FCS_CUDA(launch_task_counts(geo->d, prm->d, *particles, lo, hi, k0, k1, first_event, w, tmp, n_particles,
+                                  cfg.energy_interp, L));
+      if (size_mid_call) {
+        FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
+        FCS_CUDA(cudaStreamSynchronize(s));
+        FCS_TRY(ws_reserve_hits(ws, ws->h_sizes->n_hits, FCS_MODE_ATOMIC));
+        w = ws->view();
+      }
+      FCS_CUDA(launch_task_finish(w, nullptr, size_mid_call ? 1 : 0, n_particles * geo->d.n_layers, L));
+      const float* g = dL_dcells + (int64_t)lo * geo->d.n_cells;
+      FCS_CUDA(launch_hits_grad(geo->d, prm->d, w, lo, k0, k1, first_event, hc, g, ws->grad_acc, ws->grad_touched, L));
+      FCS_CUDA(launch_recheck_grad(geo->d, prm->d, w, lo, k0, k1, first_event, g, ws->grad_acc, ws->grad_touched, L));
+      FCS_CUDA(launch_dependent(k_range_end, 1, 1, 0, s, ws->d_sizes));
     }
-    FCS_CUDA(launch_task_finish(w, nullptr, cfg.sync ? 1 : 0, n_particles * geo->d.n_layers, L));
-    const float* g = dL_dcells + (int64_t)lo * geo->d.n_cells;
-    FCS_CUDA(launch_hits_grad(geo->d, prm->d, w, lo, k0, k1, first_event, hc, g, ws->grad_acc, ws->grad_touched, L));
-    FCS_CUDA(launch_recheck_grad(geo->d, prm->d, w, lo, k0, k1, first_event, g, ws->grad_acc, ws->grad_touched, L));
-    FCS_CUDA(launch_dependent(k_range_end, 1, 1, 0, s, ws->d_sizes));
+    FCS_CUDA(launch_grad_finalize(prm->d, ws->grad_acc, ws->grad_touched, d_frac, d_shape_w, L));
+    FCS_CUDA(cudaGetLastError());
+    ws->grad_dirty = false;
+    if (!cfg.sync) return ok();
+    FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
+    FCS_CUDA(cudaStreamSynchronize(s));
+    if (size_mid_call || attempt > 0 || !(ws->h_sizes->flags & FCS_FLAG_HIT_CAPACITY)) break;
+    size_mid_call = true;
   }
-  FCS_CUDA(launch_grad_finalize(prm->d, ws->grad_acc, ws->grad_touched, d_frac, d_shape_w, L));
-  FCS_CUDA(cudaGetLastError());
-  ws->grad_dirty = false;
-  if (!cfg.sync) return ok();
-  FCS_CUDA(cudaMemcpyAsync(ws->h_sizes, ws->d_sizes, sizeof(Sizes), cudaMemcpyDeviceToHost, s));
-  FCS_CUDA(cudaStreamSynchronize(s));
   return status_from(*ws->h_sizes, stats);
 }
 

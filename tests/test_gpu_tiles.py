@@ -71,3 +71,25 @@ def test_table_updates(geo, prm, ogeo):
         check(dataclasses.replace(prm, shape_w=w1))
     finally:
         s.close()
+
+
+def test_backward_outgrows_workspace(geo, prm):
+    """A synchronous backward call on a workspace sized by a smaller call runs
+    again with the workspace grown: the gradients are those of a fresh one."""
+    small, big = synth.single_particle(1), synth.ttbar_like(3, 4)
+    out = []
+    for first in (small, big):
+        s = fcs.Simulator(geo, prm)
+        try:
+            g = torch.Generator("cuda").manual_seed(1)
+            dl = torch.randn((4, s.n_cells), generator=g, device="cuda")
+            s.backward(s.to_device(first), 3, dl[:first.n_events])
+            r = s.backward(s.to_device(big), 3, dl)
+            torch.cuda.synchronize()
+            assert r["status"] == 0
+            out.append((r["stats"], r["d_frac"].cpu(), r["d_shape_w"].cpu()))
+        finally:
+            s.close()
+    assert out[0][0]["n_hits"] == out[1][0]["n_hits"] > 0
+    for a, b in zip(out[0][1:], out[1][1:]):
+        torch.testing.assert_close(a, b, rtol=1e-6, atol=1e-6 * float(b.abs().max()))
