@@ -1708,7 +1708,8 @@ extern "C" int fcs_simulate_events_static(const fcs_geo* geo, const fcs_params* 
   w.rows_cap = n_events;
   w.acc_stride = geo->d.acc_stride;
   const int64_t chunks = compact_chunks(geo->d.n_cells, n_events);
-  w.ss_cap = std::max(scan_state_words(std::max({P * NL, (int64_t)n_events * geo->d.acc_stride, chunks})), chunks + 2);
+  w.ss_cap = std::max(scan_state_words(std::max({P * NL, (int64_t)n_events * geo->d.acc_stride, chunks}), false),
+                      chunks + 2);
   w.scan_state = c.take<uint64_t>(w.ss_cap);
   w.recheck = c.take<uint2>(recheck_cap);
   w.recheck_cap = recheck_cap;

@@ -301,17 +301,18 @@ struct Launch {
 cudaError_t launch_build_tables(const float* frac, const float* shape_w, int n_entries, int all, uint8_t* built,
                                 int32_t* list, int32_t* n_list, uint32_t* thr, uint32_t* guide, cudaStream_t s);
 
-// fcs_scan.cu: exclusive scan of n int64 values (n on the host or device),
-// one pass.  The state (ticket, done count, one status word per tile) is zero
-// between scans; scan_state_words(n) words hold a scan of up to n elements.
+// fcs_scan.cu: exclusive scan of n int64 values (n on the host or device, at
+// most n_max), one pass.  The state (ticket, done count, one status word per tile) is zero
+// between scans; scan_state_words(n) words hold a scan of up to n elements (with
+// small_tiles, in the small tiles that short scans take where the words allow).
 struct ScanTmp {
   uint64_t* state;    // zeroed device words: [0] tile ticket, [1] CTAs done, [2 ..] tile status
   int64_t cap_tiles;  // tiles the status words cover
   uint32_t* flags;    // device flag word of the call (FCS_FLAG_WAIT_TIMEOUT)
   int grid;           // persistent CTAs
 };
-int64_t scan_state_words(int64_t max_elements);
-cudaError_t launch_scan_i64(const int64_t* in, int64_t* out, const int64_t* n_dev, int64_t n_host,
+int64_t scan_state_words(int64_t max_elements, bool small_tiles = true);
+cudaError_t launch_scan_i64(const int64_t* in, int64_t* out, const int64_t* n_dev, int64_t n_host, int64_t n_max,
                             int64_t* total_dst, int64_t total_add_base_from_dst, ScanTmp tmp,
                             cudaStream_t s);
 // Self-test of the scan's bounded wait (a tile that never publishes): the
@@ -321,10 +322,10 @@ cudaError_t scan_wait_selftest(uint32_t* flags_out, float* ms, cudaStream_t s);
 // the inputs as it reads them.
 cudaError_t launch_scan_u32_zero(uint32_t* in, int32_t* out, int64_t n, ScanTmp tmp, cudaStream_t s);
 // The hit offsets th (exclusive scan of the tasks' hit counts tn, *n_tasks of
-// them; total to *n_hits) and the tile map gmap[g] = the task holding hit
+// them, at most n_max; total to *n_hits) and the tile map gmap[g] = the task holding hit
 // g * kGranule, for g < gmap_cap.
-cudaError_t launch_scan_hits(const int32_t* tn, int64_t* th, const int64_t* n_tasks, int64_t* n_hits, int32_t* gmap,
-                             int64_t gmap_cap, ScanTmp tmp, cudaStream_t s);
+cudaError_t launch_scan_hits(const int32_t* tn, int64_t* th, const int64_t* n_tasks, int64_t n_max, int64_t* n_hits,
+                             int32_t* gmap, int64_t gmap_cap, ScanTmp tmp, cudaStream_t s);
 
 // fcs_tasks.cu: tasks, Poisson counts and the two scans (task and hit offsets);
 // then the records' hit offsets, the tile map and the validation dumps.

@@ -395,7 +395,8 @@ __global__ void __launch_bounds__(128) k_particle_count(const ParamDev p, const 
 // counts, n = max(1, Poisson(mu)), in one pass: a task's draw runs while its
 // record is still at hand, so the records are written once and not read back.
 //
-// Building: a warp takes 32 consecutive particles, whose tasks are consecutive
+// Building: a warp takes `group` consecutive particles (32, or fewer where
+// groups of 32 would leave the SMs without warps), whose tasks are consecutive
 // too (poff), and fills them 32 at a time: lane s of a round builds the task in
 // slot s of the warp's range, so each round writes 32 consecutive 32-byte
 // records.  Each lane first lists its particle's tasks in shared memory (slot
@@ -523,7 +524,7 @@ __device__ __forceinline__ uint32_t home_region(const GeoDev& g, int l, float et
 
 __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g, const ParamDev p,
                                                                  const fcs_particles parts, int32_t ev_lo, WsDev w,
-                                                                 PhiloxRoundKeys rk, uint32_t first_event_lo) {
+                                                                 PhiloxRoundKeys rk, uint32_t first_event_lo, int group) {
   dependent_start();
   __shared__ DrawEnt s_e[2][kBuildWarps][kDrawQ];  // inversion and PTRS queues
   __shared__ uint8_t s_it[2][kBuildWarps][kDrawQ];
@@ -537,9 +538,9 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_task_build(const GeoDev g,
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   WarpQueue qi{s_e[0][wi], s_it[0][wi], 0}, qp{s_e[1][wi], s_it[1][wi], 0};
   const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t wb = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; wb < P; wb += warps * 32) {
+  for (int64_t wb = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * group; wb < P; wb += warps * group) {
     const int64_t li = wb + lane;
-    const bool have = li < P;
+    const bool have = lane < group && li < P;
     const uint4 info = have ? w.pinfo[li] : make_uint4(0u, 0u, 0u, 0u);
     const int cnt = __popc(info.z);
     int incl = cnt;
@@ -861,7 +862,7 @@ cudaError_t launch_task_counts(const GeoDev& g, const ParamDev& p, const fcs_par
   cudaError_t e = launch_dependent(k_particle_count, gp, 128, 0, L.s, p, parts, ev_lo, ev_hi, w, energy_interp, k0, k1,
                                    (uint32_t)first_event);
   if (e != cudaSuccess) return e;
-  e = launch_scan_i64(w.pcount, w.poff, &w.sizes->n_part, 0, &w.sizes->n_tasks, 0, tmp, L.s);
+  e = launch_scan_i64(w.pcount, w.poff, &w.sizes->n_part, 0, n_part_max, &w.sizes->n_tasks, 0, tmp, L.s);
   if (e != cudaSuccess) return e;
   // the build kernel loops grid-stride: one wave of resident blocks
   static std::atomic<int> occ_by_device[kMaxDevices];
@@ -873,9 +874,14 @@ cudaError_t launch_task_counts(const GeoDev& g, const ParamDev& p, const fcs_par
     occ_by_device[dev].store(occ, std::memory_order_relaxed);
   }
   const PhiloxRoundKeys rk = philox_round_keys(k0, k1);
-  const int gb = (int)std::min<int64_t>((std::max<int64_t>(n_part_max, 1) + 32 * kBuildWarps - 1) / (32 * kBuildWarps),
-                                        (int64_t)L.num_sms * occ);
-  e = launch_dependent(k_task_build, gb, 32 * kBuildWarps, 0, L.s, g, p, parts, ev_lo, w, rk, (uint32_t)first_event);
+  // particles per warp: a group's rounds run one after the other, so groups
+  // shrink until each SM has 16 warps (400 particles: 24 us with 32, 10 with 4)
+  int group = 32;
+  while (group > 4 && n_part_max < (int64_t)group * L.num_sms * 16) group /= 2;
+  const int64_t warps = (std::max<int64_t>(n_part_max, 1) + group - 1) / group;
+  const int gb = (int)std::min<int64_t>((warps + kBuildWarps - 1) / kBuildWarps, (int64_t)L.num_sms * occ);
+  e = launch_dependent(k_task_build, gb, 32 * kBuildWarps, 0, L.s, g, p, parts, ev_lo, w, rk, (uint32_t)first_event,
+                       group);
   if (e != cudaSuccess) return e;
   // the FP64 pipe is narrow: one warp per block spreads the few deferred draws
   // over every SM
@@ -883,7 +889,8 @@ cudaError_t launch_task_counts(const GeoDev& g, const ParamDev& p, const fcs_par
                        p.lfact64, p.n_lfact);
   if (e != cudaSuccess) return e;
   // the scan counts the tasks actually written (n_tasks <= task_cap by construction)
-  return launch_scan_hits(w.tn, w.th, &w.sizes->n_tasks, &w.sizes->n_hits, w.gmap, w.gmap_cap, tmp, L.s);
+  return launch_scan_hits(w.tn, w.th, &w.sizes->n_tasks, n_part_max * p.NL, &w.sizes->n_hits, w.gmap, w.gmap_cap, tmp,
+                          L.s);
 }
 
 cudaError_t launch_task_finish(WsDev w, const fcs_debug* dbg, int fill_map, int64_t n_task_max, const Launch& L) {
