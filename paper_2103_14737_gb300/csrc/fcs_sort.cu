@@ -229,51 +229,94 @@ __device__ __forceinline__ const float* event_ehit(const float* __restrict__ tas
   return task_ehit + base[(uint32_t)c / acc_stride];
 }
 
-// One thread per cell: segments of up to 8 records (92 % of the hit cells of
-// pile-up events) are sorted as a copy in registers, with nothing written
-// back, and folded; segments of 9 to 16 and of 17 to kThreadSortMax records
-// are listed for the two k_det_fold_mid kernels and longer ones for
-// k_det_fold_big, so that the warps of each kernel run one path.  The list
-// array holds three lists, from its start, a third in and two thirds in: a
-// listed cell has at least 9 records, so each list fits its third.
-__global__ void __launch_bounds__(256) k_det_fold(const uint32_t* __restrict__ recs,
+// Segments of up to 8 records (92 % of the hit cells of pile-up events) are
+// sorted as a copy in registers, with nothing written back, and folded;
+// segments of 9 to 16 and of 17 to kThreadSortMax records are listed for the
+// two k_det_fold_mid kernels and longer ones for k_det_fold_big, so that the
+// warps of each kernel run one path.  The list array holds three lists, from
+// its start, a third in and two thirds in: a listed cell has at least 9 records,
+// so each list fits its third.
+//
+// Most cells are empty (half of a pile-up event's, 95 % of a hard scatter's),
+// and a warp that folds 32 neighbouring cells folds for the few that are not.
+// So a warp reads the offsets of 64 cells at a time, puts the cells to fold into
+// a queue of its own and folds 32 of them whenever it holds that many: 33 hard
+// scatters 52 to 26 us, 64 pile-up events 137 to 108 (256 cells at a time, 5 CTAs
+// per SM: 28 and 123).
+constexpr int kFoldWarps = 8, kFoldLoads = 2;
+constexpr int kFoldQueue = 32 * (kFoldLoads + 1);  // < 32 left after the folds + the new
+
+struct FoldEnt {
+  uint32_t c;     // cell
+  int32_t a, n;   // its segment
+};
+
+__global__ void __launch_bounds__(32 * kFoldWarps, 6) k_det_fold(const uint32_t* __restrict__ recs,
                                                   const int32_t* __restrict__ cell_off, int64_t n_cells_all, Sizes* sz,
                                                   int64_t cap, uint32_t acc_stride, const int64_t* __restrict__ base,
                                                   const float* __restrict__ task_ehit, double* __restrict__ acc,
                                                   int64_t* __restrict__ lists) {
   dependent_start();
+  __shared__ FoldEnt s_q[kFoldWarps][kFoldQueue];
   if (sz->flags & (FCS_FLAG_HIT_CAPACITY | FCS_FLAG_KEY_BITS)) return;
   const int lane = threadIdx.x & 31;
+  FoldEnt* const queue = s_q[threadIdx.x >> 5];
   const unsigned below = (1u << lane) - 1u;
+  int held = 0;
+  const int64_t step = (int64_t)gridDim.x * kFoldWarps * 32 * kFoldLoads;
   // warp-uniform trips, so that the lists take one counter update per warp
-  for (int64_t c0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); c0 < n_cells_all;
-       c0 += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t c = c0 + lane;
-    // the segment ends (int32, as is the record count): each lane's, and the
-    // one before the warp's first cell
-    const int32_t b = c < n_cells_all ? cell_off[c] : 0;
-    const int32_t b0 = (lane == 0 && c0 > 0) ? cell_off[c0 - 1] : 0;
-    const int32_t bp = __shfl_up_sync(0xffffffffu, b, 1);
-    const int32_t a = lane ? bp : b0;
-    const int32_t n = c < n_cells_all ? min((int64_t)b, cap) - a : 0;
-    const unsigned mb = __ballot_sync(0xffffffffu, n > kThreadSortMax);
-    const unsigned m16 = __ballot_sync(0xffffffffu, n > 8 && n <= 16);
-    const unsigned m32 = __ballot_sync(0xffffffffu, n > 16 && n <= kThreadSortMax);
-    if (mb | m16 | m32) {
-      unsigned long long bb = 0, b16 = 0, b32 = 0;
-      if (lane == 0) {
-        if (mb) bb = atomicAdd((unsigned long long*)&sz->n_big, (unsigned long long)__popc(mb));
-        if (m16) b16 = atomicAdd((unsigned long long*)&sz->n_mid, (unsigned long long)__popc(m16));
-        if (m32) b32 = atomicAdd((unsigned long long*)&sz->n_mid32, (unsigned long long)__popc(m32));
-      }
-      bb = __shfl_sync(0xffffffffu, bb, 0);
-      b16 = __shfl_sync(0xffffffffu, b16, 0);
-      b32 = __shfl_sync(0xffffffffu, b32, 0);
-      if ((mb >> lane) & 1u) lists[bb + __popc(mb & below)] = c;
-      if ((m16 >> lane) & 1u) lists[cap / 3 + (int64_t)(b16 + __popc(m16 & below))] = c;
-      if ((m32 >> lane) & 1u) lists[2 * (cap / 3) + (int64_t)(b32 + __popc(m32 & below))] = c;
+  for (int64_t w0 = ((int64_t)blockIdx.x * kFoldWarps + (threadIdx.x >> 5)) * 32 * kFoldLoads; w0 < n_cells_all;
+       w0 += step) {
+    // the segment ends (int32, as is the record count) and the one before the
+    // warp's first cell
+    int32_t ends[kFoldLoads];
+#pragma unroll
+    for (int j = 0; j < kFoldLoads; ++j) {
+      const int64_t c = w0 + 32 * j + lane;
+      ends[j] = c < n_cells_all ? cell_off[c] : -1;
     }
-    if (n > 0 && n <= 8) acc[c] = fold_small<8>(recs, a, (int)n, event_ehit(task_ehit, base, c, acc_stride));
+    int32_t prev = w0 > 0 ? cell_off[w0 - 1] : 0;  // the end before the row of 32
+#pragma unroll
+    for (int j = 0; j < kFoldLoads; ++j) {
+      const int64_t c = w0 + 32 * j + lane;
+      const int32_t up = __shfl_up_sync(0xffffffffu, ends[j], 1);
+      const int32_t a = lane ? up : prev;
+      prev = __shfl_sync(0xffffffffu, ends[j], 31);
+      const int32_t n = ends[j] >= 0 ? (int32_t)(min((int64_t)ends[j], cap) - a) : 0;
+      if (!__any_sync(0xffffffffu, n > 0)) continue;
+      const unsigned mb = __ballot_sync(0xffffffffu, n > kThreadSortMax);
+      const unsigned m16 = __ballot_sync(0xffffffffu, n > 8 && n <= 16);
+      const unsigned m32 = __ballot_sync(0xffffffffu, n > 16 && n <= kThreadSortMax);
+      if (mb | m16 | m32) {
+        unsigned long long bb = 0, b16 = 0, b32 = 0;
+        if (lane == 0) {
+          if (mb) bb = atomicAdd((unsigned long long*)&sz->n_big, (unsigned long long)__popc(mb));
+          if (m16) b16 = atomicAdd((unsigned long long*)&sz->n_mid, (unsigned long long)__popc(m16));
+          if (m32) b32 = atomicAdd((unsigned long long*)&sz->n_mid32, (unsigned long long)__popc(m32));
+        }
+        bb = __shfl_sync(0xffffffffu, bb, 0);
+        b16 = __shfl_sync(0xffffffffu, b16, 0);
+        b32 = __shfl_sync(0xffffffffu, b32, 0);
+        if ((mb >> lane) & 1u) lists[bb + __popc(mb & below)] = c;
+        if ((m16 >> lane) & 1u) lists[cap / 3 + (int64_t)(b16 + __popc(m16 & below))] = c;
+        if ((m32 >> lane) & 1u) lists[2 * (cap / 3) + (int64_t)(b32 + __popc(m32 & below))] = c;
+      }
+      const bool small = n > 0 && n <= 8;
+      const unsigned ms = __ballot_sync(0xffffffffu, small);
+      if (small) queue[held + __popc(ms & below)] = FoldEnt{(uint32_t)c, a, n};
+      held += __popc(ms);
+    }
+#pragma unroll 1
+    while (held >= 32 || (held && w0 + step >= n_cells_all)) {  // (the last trip folds what is left)
+      const int cnt = min(held, 32);
+      __syncwarp();
+      if (lane < cnt) {
+        const FoldEnt e = queue[held - cnt + lane];
+        acc[e.c] = fold_small<8>(recs, e.a, e.n, event_ehit(task_ehit, base, e.c, acc_stride));
+      }
+      held -= cnt;
+    }
+    __syncwarp();
   }
 }
 
