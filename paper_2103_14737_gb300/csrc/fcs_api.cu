@@ -172,6 +172,8 @@ struct fcs_workspace {
   uint2* recheck = nullptr;
   int64_t recheck_cap = 0;
   double* acc = nullptr;  // FP64 accumulation rows
+  uint8_t* marks = nullptr;  // of the rows' touched cells (calls of sparse events)
+  int64_t marks_cap = 0;
   int64_t acc_cap = 0, rows_cap = 0;
   int32_t acc_stride = 0;
   uint64_t* scan_state = nullptr;  // zero between scans (see ScanTmp)
@@ -223,7 +225,7 @@ struct fcs_workspace {
     if (s_out) cudaStreamDestroy(s_out);
     if (scan_state2) cudaFree(scan_state2);
     void* ps[] = {d_sizes, pcount, poff, pinfo, tasks, tehit, tn, th, pdefer, gmap,
-                  recheck, acc, scan_state, keys, keys_alt, cell_off, stage, grad_acc, grad_touched};
+                  recheck, acc, marks, scan_state, keys, keys_alt, cell_off, stage, grad_acc, grad_touched};
     for (void* p : ps)
       if (p) cudaFree(p);
     if (h_sizes) cudaFreeHost(h_sizes);
@@ -299,6 +301,7 @@ int ws_reserve_static(fcs_workspace* ws, const fcs_geo* geo, int64_t P, int32_t 
     ws->rows_cap = std::max(rows, 1);
     ws->acc_stride = stride;
   }
+  FCS_TRY(grow(&ws->marks, &ws->marks_cap, ((int64_t)std::max(rows, 1) * stride) >> kMarkShift, true));
   const int64_t chunks = compact_chunks(geo->d.n_cells, std::max(rows, 1));
   // scan state for the largest array any scan of a call covers, and a status
   // word per compaction chunk (zeroed; the scans and the compaction leave it
@@ -445,7 +448,28 @@ struct CallArgs {
   int64_t capacity;
   const fcs_debug* dbg;
   cudaStream_t s;
+  bool sparse = false;  // see sparse_events
 };
+
+// Whether a call marks what its deposits touch and compacts only that: events
+// of few particles touch a few of a row's 46 chunks, and the compaction of whole
+// rows, 1.5 MB each, is most of the call.  From 32 rows on: below, the
+// compaction is a chain of latencies either way (8 rows of one particle 14 us by
+// both, 16 rows 21 and 16, 32 rows 31 and 17).  Up to 8 particles an event on
+// average: the marks cost the hit kernel up to 4 %, which grows with the hits,
+// while the gain shrinks as the rows fill (whole call, us, reading all and
+// marked: 500 x 1 of 65 GeV 366 and 108, 500 x 8 486 and 276, 500 x 32 746 and
+// 655, 64 x 8 153 and 134, 64 x 100 289 and 310; of 1 TeV 64 x 16 546 and 556; of
+// 4 TeV 64 x 4 884 and 879).  Only the hit kernel's default shape marks.
+constexpr int32_t kSparseRows = 32;
+constexpr int64_t kSparseParticles = 8;
+bool sparse_events(const CallArgs& a, int32_t rows) {
+  const fcs_config& c = a.cfg;
+  const bool dumps = a.dbg && (a.dbg->hit_cell || a.dbg->hit_bin);
+  return c.mode == FCS_MODE_ATOMIC && c.batched == 1 && (c.block == 0 || c.block == 128) && !a.cells_out && !dumps &&
+         rows >= kSparseRows && a.n_particles <= kSparseParticles * a.n_events &&
+         a.geo->d.acc_stride >> kMarkShift <= kMaxRowMarks;
+}
 
 // Stage events: inside a stream capture they must be external events to
 // become event-record nodes of the graph; outside a capture plain records.
@@ -496,6 +520,7 @@ int enqueue_range_hits(const CallArgs& a, int32_t ev_lo, int32_t ev_hi, int32_t 
   auto view = [&]() {
     WsDev v = ws->view();
     v.acc = ws->acc + acc_row0 * ws->acc_stride;
+    v.marks = a.sparse ? ws->marks : nullptr;
     return v;
   };
   WsDev w = view();
@@ -547,6 +572,10 @@ int enqueue_range_reduce(const CallArgs& a, WsDev w, int32_t ev_lo, int32_t rows
                          cudaStream_t s, int max_ctas = 0) {
   fcs_workspace* ws = a.ws;
   const Launch L{s, ws->num_sms};
+  if (w.marks) {
+    FCS_CUDA(launch_compact_sparse(a.geo->d, w, rows, ev_lo, tmp, a.cell_ids, a.cell_E, a.event_offsets_out, a.capacity, L));
+    return FCS_OK;
+  }
   if (a.cfg.mode == FCS_MODE_DETERMINISTIC)
     FCS_CUDA(launch_det_reduce(a.geo->d, w, rows, key_task_bits, ws->cell_off, a.parts.event_offsets, ev_lo, tmp, L));
   FCS_CUDA(launch_compact(a.geo->d, w, rows, ev_lo, tmp, a.cells_out, a.cell_ids, a.cell_E, a.event_offsets_out,
@@ -1278,6 +1307,7 @@ int fcs_simulate_events(const fcs_geo* geo, const fcs_params* prm, fcs_workspace
     return set_err(FCS_E_RANGE, "deterministic mode: (cell, task) keys exceed 63 bits; use smaller waves or split the batch");
   CallArgs a{geo, prm, ws, *particles, n_particles, n_events, seed, first_event, cfg, cells_out,
              cell_ids, cell_E, event_offsets_out, capacity, dbg, s};
+  a.sparse = sparse_events(a, rows);
   const HitCfg hc = hit_cfg(cfg);
   if (cfg.timing) FCS_TRY(ensure_timing_events(ws, n_ranges(cfg, n_events)));
   else ws->timed_ranges = 0;
@@ -1310,6 +1340,7 @@ int fcs_simulate_events(const fcs_geo* geo, const fcs_params* prm, fcs_workspace
     put(&ws->gmap, sizeof(void*));
     put(&ws->recheck, sizeof(void*));
     put(&ws->acc, sizeof(void*));
+    put(&ws->marks, sizeof(void*));
     put(&ws->keys, sizeof(void*));
     put(&ws->cell_off, sizeof(void*));
     if (!ws->graph || key != ws->graph_key) {

@@ -206,6 +206,160 @@ __global__ void __launch_bounds__(kCThreads, kCtasPerSm) k_compact_one(const Com
   }
 }
 
+constexpr int kSparseCtas = 8;       // per SM
+constexpr int kSparseParts = 304;    // parts wanted of all rows
+
+// Rows of sparse events (some particles each): a CTA takes a part of a row (all
+// of it from 304 rows on), in ticket order, lists the 64-cell groups that the
+// range's deposits marked there, gives each warp a run of them, and reads only
+// those: once to count and again, from the caches and only where the run is
+// too long for the warp's registers, to write the pairs and zero the cells.
+//
+// k_compact_one reads every row: 500 single electrons leave 27,782 hit cells in
+// 753 MB, and the look-backs run over 23,000 chunks.  Here the marks (1.5 MB)
+// and the marked groups are read, and the look-backs run over 500 parts; what
+// is left is the chain ticket, marks, groups, look-back, pairs of one CTA.
+// Rows x particles of 65 GeV:   16 x 1   64 x 1   500 x 1   500 x 8   16384 x 1
+//   k_compact_one (us)            21       47       275       297       8600
+//   here                          16       18        21        90        300
+// (marks of 4096 cells 133 us at 500 x 1; parts for 608 CTAs of 4 an SM, 8
+// groups in flight 25.)
+__global__ void __launch_bounds__(kCThreads, kSparseCtas) k_compact_sparse(const CompactArgs A, uint8_t* __restrict__ marks) {
+  dependent_start();
+  __shared__ uint16_t s_list[kMaxRowMarks];  // the part's marked groups, in order
+  __shared__ int s_w[kCWarps];               // per warp: marked groups listed; then hit cells
+  __shared__ unsigned long long s_ticket;
+  __shared__ int64_t s_base;
+  __shared__ int s_last;
+  constexpr int kSeg = kMaxRowMarks / kCThreads;  // marks of a lane, at most
+  constexpr int kLoads = 2;                       // groups of a warp in flight
+  unsigned long long* ticket = reinterpret_cast<unsigned long long*>(A.state);
+  unsigned long long* done = ticket + 1;
+  uint64_t* status = A.state + 2;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned below = (1u << lane) - 1u;
+  const int row_marks = A.stride >> kMarkShift;
+  const int part_marks = (row_marks + A.cpr - 1) / A.cpr;
+  const int seg = (part_marks + kCWarps - 1) / kCWarps;  // marks of a warp
+  int64_t n_t = A.n_chunks;                              // parts
+  if (n_t > A.cap_tiles) {  // the workspace sizes the state for more: never
+    if (tid == 0) atomicOr(A.flags, (uint32_t)FCS_FLAG_WAIT_TIMEOUT);
+    n_t = 0;
+  }
+  while (true) {
+    if (tid == 0) s_ticket = atomicAdd(ticket, 1ull);
+    __syncthreads();
+    const int64_t t = (int64_t)s_ticket;
+    if (t >= n_t) break;
+    const int64_t row = t / A.cpr;
+    const int mark0 = (int)(t % A.cpr) * part_marks;
+    double2* const cells = reinterpret_cast<double2*>(A.acc + row * A.stride) + lane;
+    {
+      const int first = mark0 + warp * seg;
+      const int n = min(seg, min(mark0 + part_marks, row_marks) - first);
+      uint8_t* const mine = marks + row * row_marks + first + lane;
+      bool on[kSeg];
+#pragma unroll
+      for (int j = 0; j < kSeg; ++j) on[j] = 32 * j + lane < n && mine[32 * j] != 0;
+      int cnt = 0;
+#pragma unroll
+      for (int j = 0; j < kSeg; ++j) {
+        cnt += __popc(__ballot_sync(0xffffffffu, on[j]));
+        if (on[j]) mine[32 * j] = 0;
+      }
+      if (lane == 0) s_w[warp] = cnt;
+      __syncthreads();
+      int at = 0;
+      for (int w = 0; w < warp; ++w) at += s_w[w];
+#pragma unroll
+      for (int j = 0; j < kSeg; ++j) {
+        const unsigned m = __ballot_sync(0xffffffffu, on[j]);
+        if (on[j]) s_list[at + __popc(m & below)] = (uint16_t)(first + 32 * j + lane);
+        at += __popc(m);
+      }
+    }
+    int listed = 0;
+#pragma unroll
+    for (int w = 0; w < kCWarps; ++w) listed += s_w[w];
+    __syncthreads();  // the list is written, s_w is read
+    const int run = (listed + kCWarps - 1) / kCWarps;
+    const int lo = warp * run, hi = min(listed, lo + run);
+    double2 v[kLoads];
+    auto load = [&](int k) {
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j) v[j] = k + j < hi ? cells[32 * s_list[k + j]] : make_double2(0.0, 0.0);
+    };
+    int n = 0;  // the warp's hit cells
+    for (int k = lo; k < hi; k += kLoads) {
+      load(k);
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j)
+        n += __popc(__ballot_sync(0xffffffffu, acc_nonzero(v[j].x))) +
+             __popc(__ballot_sync(0xffffffffu, acc_nonzero(v[j].y)));
+    }
+    if (lane == 0) s_w[warp] = n;
+    __syncthreads();
+    if (warp == 0) {  // publish, look back, publish the prefix
+      int total = 0;
+#pragma unroll
+      for (int w = 0; w < kCWarps; ++w) total += s_w[w];
+      int64_t excl;
+      if (t == 0) {
+        excl = *A.total_dst;
+      } else {
+        if (lane == 0) atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagAgg | (uint64_t)total);
+        excl = look_back(status, t, A.flags);
+      }
+      if (lane == 0) {
+        atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagPrefix | (uint64_t)(excl + total));
+        s_base = excl;
+        if (mark0 == 0 && A.event_offsets_out) A.event_offsets_out[A.ev_lo + row] = excl;
+        if (t == n_t - 1) *A.total_dst = excl + total;
+      }
+    }
+    __syncthreads();
+    int64_t pos = s_base;
+    for (int w = 0; w < warp; ++w) pos += s_w[w];
+    for (int k = lo; k < hi; k += kLoads) {
+      if (hi - lo > kLoads) load(k);
+#pragma unroll
+      for (int j = 0; j < kLoads; ++j) {
+        const bool nx = acc_nonzero(v[j].x), ny = acc_nonzero(v[j].y);
+        const unsigned mx = __ballot_sync(0xffffffffu, nx), my = __ballot_sync(0xffffffffu, ny);
+        if (!(mx | my)) continue;
+        const int group = s_list[k + j];
+        if (nx || ny) cells[32 * group] = make_double2(0.0, 0.0);
+        int64_t p = pos + __popc(mx & below) + __popc(my & below);
+        const int c = (group << kMarkShift) + 2 * lane;
+        if (nx && p < A.capacity && A.cell_ids) {
+          A.cell_ids[p] = c;
+          A.cell_E[p] = acc_to_f32(v[j].x);
+        }
+        p += nx ? 1 : 0;
+        if (ny && p < A.capacity && A.cell_ids) {
+          A.cell_ids[p] = c + 1;
+          A.cell_E[p] = acc_to_f32(v[j].y);
+        }
+        pos += __popc(mx) + __popc(my);
+      }
+    }
+    __syncthreads();  // the shared arrays are reused
+  }
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1ull) == (unsigned long long)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    for (int64_t i = tid; i < n_t; i += kCThreads) status[i] = 0;
+    if (tid == 0) {
+      *ticket = 0;
+      *done = 0;
+    }
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, float* cells_out,
@@ -228,6 +382,18 @@ cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo
     return cudaGetLastError();
   }
   return launch_dependent(kernel, grid, kCThreads, 0, L.s, A);
+}
+
+cudaError_t launch_compact_sparse(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, int32_t* cell_ids,
+                                  float* cell_E, int64_t* event_offsets_out, int64_t capacity, const Launch& L) {
+  if (rows <= 0) return cudaSuccess;
+  // (no more parts than the row has chunks: the scan state's size)
+  const int parts = std::max(1, std::min((g.n_cells + kChunk - 1) / kChunk, kSparseParts / rows));
+  const int64_t n_parts = (int64_t)rows * parts;
+  const int grid = (int)std::min<int64_t>(n_parts, (int64_t)L.num_sms * kSparseCtas);
+  const CompactArgs A{w.acc, g.n_cells, g.acc_stride, parts, ev_lo, 0, n_parts, tmp.state, tmp.cap_tiles, tmp.flags,
+                      &w.sizes->nnz_total, nullptr, cell_ids, cell_E, event_offsets_out, capacity};
+  return launch_dependent(k_compact_sparse, grid, kCThreads, 0, L.s, A, w.marks);
 }
 
 int64_t compact_chunks(int32_t n_cells, int32_t rows) {

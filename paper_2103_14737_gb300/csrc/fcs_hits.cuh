@@ -433,6 +433,7 @@ __device__ __forceinline__ void deposit_single(const HitKParams& kp, int32_t eve
   const int64_t row = event - kp.ev_lo;
   if (mode == kModeAtomic) {
     acc_add(kp.w.acc + row * kp.g.acc_stride + cell, Ehit);
+    if (kp.w.marks) set_mark(kp.w.marks + ((row * kp.g.acc_stride + cell) >> kMarkShift));
   } else if (mode == kModeGrad) {
     const float v = __fmul_rn(Ehit, __ldg(kp.grad_in + row * kp.g.n_cells + cell));
     atomicAdd(kp.grad_acc + ((int64_t)entry << 7) + bin, (double)v);
@@ -498,7 +499,10 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
       grad_add(kp, ((uint32_t)T.entry() << 7) | (uint32_t)bin,
                __fmul_rn(Ehit, __ldg(kp.grad_in + row * kp.g.n_cells + c)));
   } else if constexpr (MODE == kModeAtomic) {
-    if (ok) acc_add(w.acc + row * kp.g.acc_stride + c, Ehit);
+    if (ok) {
+      acc_add(w.acc + row * kp.g.acc_stride + c, Ehit);
+      if (w.marks) set_mark(w.marks + ((row * kp.g.acc_stride + c) >> kMarkShift));
+    }
   } else {
     // records as emit_records writes them, in slots of their own
     const int lane = threadIdx.x & 31;
@@ -545,6 +549,7 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
 //   598     a warp's own tickets and passes instead of CTA tiles
 //   571     two steps in flight; 9 CTAs of 128 threads per SM at 56 registers
 //           (10 at 48: 596, 8 at 64: 571, one step in flight: 600)
+// SPARSE: the deposits set w.marks.
 // (Finishing the searches in the loop with two more loads: 610.  Without any
 // put-off hit, wrongly, it would be 500.)
 //
@@ -552,7 +557,7 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
 // fcs_debug (a separate instantiation, so that the production kernel carries
 // none of their code).
 constexpr int hits_min_ctas(int block) { return 9 * 128 / block; }
-template <int BLOCK, int MODE, bool DBG>
+template <int BLOCK, int MODE, bool DBG, bool SPARSE>
 __global__ void __launch_bounds__(BLOCK, hits_min_ctas(BLOCK)) k_hits(const __grid_constant__ HitKParams kp) {
   dependent_start();
   constexpr bool DET = MODE == kModeDet;
@@ -678,8 +683,10 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(BLOCK)) k_hits(const __gr
               m & (kp.key32 ? __match_any_sync(kAll, (f.cell << 5) | (uint32_t)d.tl)
                             : __match_any_sync(kAll, ((unsigned long long)(uint32_t)d.tl << 32) | f.cell));
           if constexpr (!DET) {
-            if (ok && (peers & lanes_below) == 0u)  // the group's first lane deposits
+            if (ok && (peers & lanes_below) == 0u) {  // the group's first lane deposits
               acc_add(w.acc + f.cell, __fmul_rn((float)__popc(peers), T.Ehit));
+              if constexpr (SPARSE) set_mark(w.marks + (f.cell >> kMarkShift));
+            }
           } else {
             const unsigned long long gkey =
                 ((unsigned long long)f.cell << kp.key_task_bits) | (unsigned long long)(t0 + d.tl);

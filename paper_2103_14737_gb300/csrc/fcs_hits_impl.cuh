@@ -26,12 +26,12 @@ static inline HitKParams make_hit_params(const GeoDev& g, const ParamDev& p, WsD
   return kp;
 }
 
-template <int BLOCK, int MODE, bool DBG>
+template <int BLOCK, int MODE, bool DBG, bool SPARSE = false>
 static cudaError_t launch_hits_kernel(const HitKParams& kp, const Launch& L) {
   static int occ = -1;  // resident CTAs per SM of this instantiation
   if (occ < 0) {
     int o = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_hits<BLOCK, MODE, DBG>, BLOCK, 0);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_hits<BLOCK, MODE, DBG, SPARSE>, BLOCK, 0);
     if (e != cudaSuccess) return e;
     occ = o < 1 ? 1 : o;
   }
@@ -41,7 +41,7 @@ static cudaError_t launch_hits_kernel(const HitKParams& kp, const Launch& L) {
     grid = (kp.h_hi - kp.h_lo + per_cta - 1) / per_cta;
     if (grid <= 0) return cudaSuccess;
   }
-  return launch_dependent(k_hits<BLOCK, MODE, DBG>, grid, BLOCK, 0, L.s, kp);
+  return launch_dependent(k_hits<BLOCK, MODE, DBG, SPARSE>, grid, BLOCK, 0, L.s, kp);
 }
 
 // The validation dumps run in their own instantiation (no gradient-mode dumps).
@@ -49,6 +49,9 @@ template <int BLOCK, int MODE>
 static cudaError_t launch_hits_block(const HitKParams& kp, const Launch& L) {
   if constexpr (MODE != kModeGrad) {
     if (kp.dbg_hit_cell || kp.dbg_hit_bin) return launch_hits_kernel<BLOCK, MODE, true>(kp, L);
+  }
+  if constexpr (MODE == kModeAtomic && BLOCK == 128) {
+    if (kp.w.marks) return launch_hits_kernel<BLOCK, MODE, false, true>(kp, L);
   }
   return launch_hits_kernel<BLOCK, MODE, false>(kp, L);
 }

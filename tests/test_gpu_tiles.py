@@ -93,3 +93,51 @@ def test_backward_outgrows_workspace(geo, prm):
     assert out[0][0]["n_hits"] == out[1][0]["n_hits"] > 0
     for a, b in zip(out[0][1:], out[1][1:]):
         torch.testing.assert_close(a, b, rtol=1e-6, atol=1e-6 * float(b.abs().max()))
+
+
+@pytest.mark.parametrize("n_events, share", [(32, 1), (33, 8), (310, 2), (64, 0), (305, -1)])
+def test_sparse_events(geo, prm, ogeo, n_events, share):
+    """Calls of at least 32 events and at most 8 particles an event read back
+    only the cells that their deposits marked: the same pairs as a call that
+    reads every cell, over empty events, an event with every particle (-1),
+    event ranges, graphs and outputs that are too small, and rows left zero."""
+    rng = np.random.default_rng(n_events)
+    n = max(share, 1) * n_events
+    off = np.arange(n_events + 1, dtype=np.int64) * share if share > 0 else np.where(
+        np.arange(n_events + 1) > (n_events // 2 if share < 0 else 0), n, 0).astype(np.int64)
+    if share == 0:  # every second event empty
+        off = np.minimum((np.arange(n_events + 1) + 1) // 2 * 2, n).astype(np.int64)
+    parts = synth.Particles(rng.integers(0, 3, n).astype(np.int32), rng.uniform(1e3, 1e5, n).astype(np.float32),
+                            rng.uniform(-5.2, 5.2, n).astype(np.float32), rng.uniform(-3.2, 3.2, n).astype(np.float32),
+                            off)
+    ref = O.simulate(ogeo, O.OracleParams(prm), parts, seed=4).cells64
+    s = fcs.Simulator(geo, prm)
+    try:
+        d = s.to_device(parts)
+
+        def check(r, n_read=None):
+            eo = r["event_offsets"].cpu().numpy()
+            nnz = int(eo[-1]) if n_read is None else n_read
+            ids, E = r["cell_ids"][:nnz].cpu().numpy(), r["cell_E"][:nnz].cpu().numpy()
+            ev, cell = np.nonzero(ref)
+            assert np.array_equal(eo, np.searchsorted(ev, np.arange(n_events + 1)))
+            assert np.array_equal(ids, cell[:nnz])
+            np.testing.assert_allclose(E, ref[ev, cell][:nnz], rtol=1e-5)
+
+        general = s.simulate(d, 4, block=256)  # reads every cell
+        check(general)
+        check(s.simulate(d, 4))
+        check(s.simulate(d, 4, wave_events=40))
+        nnz = int(general["event_offsets"][-1])
+        small = s.simulate(d, 4, capacity=nnz - 3, check=False)
+        assert small["status"] == fcs.FCS_E_RANGE
+        check(small, nnz - 3)
+        out = {k: general[k] for k in ("cell_ids", "cell_E", "event_offsets")}
+        for _ in range(2):  # captured, replayed
+            out["cell_ids"].fill_(-1)
+            s.simulate(d, 4, sync=0, use_graph=1, outputs=out)
+            torch.cuda.synchronize()
+            check(out)
+        check(s.simulate(d, 4, block=256))  # the rows were left zero
+    finally:
+        s.close()
