@@ -520,7 +520,7 @@ int enqueue_range_hits(const CallArgs& a, int32_t ev_lo, int32_t ev_hi, int32_t 
   auto view = [&]() {
     WsDev v = ws->view();
     v.acc = ws->acc + acc_row0 * ws->acc_stride;
-    v.marks = a.sparse ? ws->marks : nullptr;
+    v.marks = a.sparse ? ws->marks + acc_row0 * (ws->acc_stride >> kMarkShift) : nullptr;
     return v;
   };
   WsDev w = view();
@@ -796,6 +796,7 @@ int host_waves(const fcs_geo* geo, const fcs_params* prm, fcs_workspace* ws, con
   put(&m_oout, sizeof(m_oout));
   put(&capacity, sizeof(capacity));
   put(&view, sizeof(view));
+  put(&ws->marks, sizeof(void*));
   put(&ws->acc_stride, sizeof(ws->acc_stride));
   put(&ws->scan_state, sizeof(void*));
   put(&ws->ss_cap, sizeof(ws->ss_cap));
@@ -810,6 +811,7 @@ int host_waves(const fcs_geo* geo, const fcs_params* prm, fcs_workspace* ws, con
     FCS_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     CallArgs a{geo, prm, ws, dparts, n_particles, n_events, seed, first_event, cfg, nullptr,
                m_ids, m_cE, m_oout, capacity, nullptr, cs};
+    a.sparse = sparse_events(a, n_events);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     int rc = FCS_OK;

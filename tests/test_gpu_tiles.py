@@ -124,7 +124,7 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             assert np.array_equal(ids, cell[:nnz])
             np.testing.assert_allclose(E, ref[ev, cell][:nnz], rtol=1e-5)
 
-        general = s.simulate(d, 4, block=256)  # reads every cell
+        general = s.simulate(d, 4, block=256, capacity=1 << 18)  # reads every cell
         check(general)
         check(s.simulate(d, 4))
         check(s.simulate(d, 4, wave_events=40))
@@ -138,6 +138,13 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             s.simulate(d, 4, sync=0, use_graph=1, outputs=out)
             torch.cuda.synchronize()
             check(out)
+        pin = [torch.as_tensor(a).pin_memory() for a in (parts.type, parts.E, parts.eta, parts.phi, parts.event_offsets)]
+        host = {k: torch.zeros(v.shape, dtype=v.dtype).pin_memory() for k, v in out.items()}
+        for _ in range(2):  # host buffers, in waves of events
+            host["cell_ids"].fill_(-1)
+            fcs.fcs_simulate_events_host(s.geo, s.prm, s.ws, *(a.numpy() for a in pin), 4, 0, fcs.make_config(),
+                                         *(host[k].numpy() for k in ("cell_ids", "cell_E", "event_offsets")))
+            check(host)
         check(s.simulate(d, 4, block=256))  # the rows were left zero
     finally:
         s.close()
