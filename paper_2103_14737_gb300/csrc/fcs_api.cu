@@ -460,7 +460,8 @@ struct CallArgs {
 // while the gain shrinks as the rows fill (whole call, us, reading all and
 // marked: 500 x 1 of 65 GeV 366 and 108, 500 x 8 486 and 276, 500 x 32 746 and
 // 655, 64 x 8 153 and 134, 64 x 100 289 and 310; of 1 TeV 64 x 16 546 and 556; of
-// 4 TeV 64 x 4 884 and 879).  Only the hit kernel's default shape marks.
+// 4 TeV 64 x 4 884 and 879; from and to host buffers, in waves: 500 x 1 1687 and
+// 196, 64 x 8 358 and 195).  Only the hit kernel's default shape marks.
 constexpr int32_t kSparseRows = 32;
 constexpr int64_t kSparseParticles = 8;
 bool sparse_events(const CallArgs& a, int32_t rows) {
@@ -729,8 +730,12 @@ int enqueue_waves(const CallArgs& a, const int32_t* type, const float* E, const 
     // the compaction runs beside the next wave on a third of the SMs: its
     // stores over the CPU-GPU link need few CTAs to keep the link busy, and
     // the next wave's kernels keep the rest (a quarter starved the link on
-    // small calls; half slowed the next wave on large ones)
-    FCS_TRY(enqueue_range_reduce(a, w, bnd[k], bnd[k + 1] - bnd[k], key_task_bits, tmp2, s_out, ws->num_sms / 3));
+    // small calls; half slowed the next wave on large ones).  The last wave's
+    // runs alone, two CTAs to an SM: 64 t-tbar events of 12,500 hit cells 468
+    // to 415 us, 600 events of 38,900 cells 3721 to 3400 (one an SM 425 and
+    // 3402; four 418 and 3474: the stores get in each other's way)
+    FCS_TRY(enqueue_range_reduce(a, w, bnd[k], bnd[k + 1] - bnd[k], key_task_bits, tmp2, s_out,
+                                 k + 1 == nw ? 2 * ws->num_sms : ws->num_sms / 3));
   }
   k_call_end<<<1, 1, 0, s_out>>>(ws->d_sizes, a.event_offsets_out, a.n_events, a.capacity, a.cell_ids ? 1 : 0,
                                   ws->h_sizes);
