@@ -370,6 +370,7 @@ __global__ void __launch_bounds__(kRangeThreads) k_range_begin(Sizes* s, const i
   s->n_big = 0;
   s->n_mid = 0;
   s->n_mid32 = 0;
+  s->seg_alloc = 0;
   s->n_pdefer = 0;
   s->n_pdefer_ptrs = 0;
   s->queue = 0;
@@ -461,14 +462,17 @@ struct CallArgs {
 // marked: 500 x 1 of 65 GeV 366 and 108, 500 x 8 486 and 276, 500 x 32 746 and
 // 655, 64 x 8 153 and 134, 64 x 100 289 and 310; of 1 TeV 64 x 16 546 and 556; of
 // 4 TeV 64 x 4 884 and 879; from and to host buffers, in waves: 500 x 1 1687 and
-// 196, 64 x 8 358 and 195).  Only the hit kernel's default shape marks.
+// 196, 64 x 8 358 and 195).  Deterministic calls, which also scan and fold by
+// cells, gain up to twice that: 500 x 1 942 and 153, 500 x 8 1102 and 498, 64 x 16
+// 305 and 271, 64 x 32 333 and 334.  Only the hit kernel's default shape marks.
 constexpr int32_t kSparseRows = 32;
-constexpr int64_t kSparseParticles = 8;
+constexpr int64_t kSparseParticles = 8, kSparseParticlesDet = 16;
 bool sparse_events(const CallArgs& a, int32_t rows) {
   const fcs_config& c = a.cfg;
+  const int64_t limit = c.mode == FCS_MODE_DETERMINISTIC ? kSparseParticlesDet : kSparseParticles;
   const bool dumps = a.dbg && (a.dbg->hit_cell || a.dbg->hit_bin);
-  return c.mode == FCS_MODE_ATOMIC && c.batched == 1 && (c.block == 0 || c.block == 128) && !a.cells_out && !dumps &&
-         rows >= kSparseRows && a.n_particles <= kSparseParticles * a.n_events &&
+  return c.batched == 1 && (c.block == 0 || c.block == 128) && !a.cells_out && !dumps &&
+         rows >= kSparseRows && a.n_particles <= limit * a.n_events &&
          a.geo->d.acc_stride >> kMarkShift <= kMaxRowMarks;
 }
 
@@ -573,12 +577,12 @@ int enqueue_range_reduce(const CallArgs& a, WsDev w, int32_t ev_lo, int32_t rows
                          cudaStream_t s, int max_ctas = 0) {
   fcs_workspace* ws = a.ws;
   const Launch L{s, ws->num_sms};
+  if (a.cfg.mode == FCS_MODE_DETERMINISTIC)
+    FCS_CUDA(launch_det_reduce(a.geo->d, w, rows, key_task_bits, ws->cell_off, a.parts.event_offsets, ev_lo, tmp, L));
   if (w.marks) {
     FCS_CUDA(launch_compact_sparse(a.geo->d, w, rows, ev_lo, tmp, a.cell_ids, a.cell_E, a.event_offsets_out, a.capacity, L));
     return FCS_OK;
   }
-  if (a.cfg.mode == FCS_MODE_DETERMINISTIC)
-    FCS_CUDA(launch_det_reduce(a.geo->d, w, rows, key_task_bits, ws->cell_off, a.parts.event_offsets, ev_lo, tmp, L));
   FCS_CUDA(launch_compact(a.geo->d, w, rows, ev_lo, tmp, a.cells_out, a.cell_ids, a.cell_E, a.event_offsets_out,
                           a.capacity, max_ctas, L));
   return FCS_OK;

@@ -382,6 +382,7 @@ struct RecordChunk {
   int fill = kRecordChunk;  // no chunk yet
 };
 
+template <bool SPARSE>
 __device__ __forceinline__ unsigned emit_records(bool ok, unsigned peers, unsigned long long gkey, uint32_t cell,
                                                  RecordChunk& ch, const WsDev& w) {
   const int lane = threadIdx.x & 31;
@@ -401,6 +402,7 @@ __device__ __forceinline__ unsigned emit_records(bool ok, unsigned peers, unsign
     if (slot < w.rec_cap) {
       w.keys[slot] = (gkey << kRecordCountBits) | (unsigned long long)(__popc(peers) - 1);
       atomicAdd(reinterpret_cast<uint32_t*>(w.acc) + cell, 1u);
+      if constexpr (SPARSE) set_mark(w.marks + (cell >> kMarkShift));
     } else {
       atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_HIT_CAPACITY);
     }
@@ -446,6 +448,7 @@ __device__ __forceinline__ void deposit_single(const HitKParams& kp, int32_t eve
       atomicAdd((unsigned long long*)&kp.w.sizes->n_records, 1ull);
       kp.w.keys[slot] = gkey << kRecordCountBits;
       atomicAdd(reinterpret_cast<uint32_t*>(kp.w.acc) + c, 1u);
+      if (kp.w.marks) set_mark(kp.w.marks + (c >> kMarkShift));
     } else {
       atomicOr(&kp.w.sizes->flags, (uint32_t)FCS_FLAG_HIT_CAPACITY);
     }
@@ -522,6 +525,7 @@ static __device__ __noinline__ void deferred_hits(const HitKParams& kp, bool hav
       if (slot < w.rec_cap) {
         w.keys[slot] = (gkey << kRecordCountBits) | (unsigned long long)(__popc(peers) - 1);
         atomicAdd(reinterpret_cast<uint32_t*>(w.acc) + cg, 1u);
+        if (w.marks) set_mark(w.marks + (cg >> kMarkShift));
       } else {
         atomicOr(&w.sizes->flags, (uint32_t)FCS_FLAG_HIT_CAPACITY);
       }
@@ -690,7 +694,7 @@ __global__ void __launch_bounds__(BLOCK, hits_min_ctas(BLOCK)) k_hits(const __gr
           } else {
             const unsigned long long gkey =
                 ((unsigned long long)f.cell << kp.key_task_bits) | (unsigned long long)(t0 + d.tl);
-            recs += emit_records(ok, peers, gkey, f.cell, chunk, w);
+            recs += emit_records<SPARSE>(ok, peers, gkey, f.cell, chunk, w);
           }
         }
         if constexpr (DBG) {

@@ -132,6 +132,7 @@ struct Sizes {
   int64_t n_pdefer;     // inversion draws deferred to FP64 in the current range (front of pdefer)
   int64_t n_pdefer_ptrs;  // PTRS draws deferred to FP64 in the current range (back of pdefer)
   unsigned long long queue;  // hit-kernel work-queue counter (tiles handed out)
+  unsigned long long seg_alloc;  // deterministic calls of sparse events: marked groups << 32 | their records
   uint32_t flags;       // fcs_device_flag bits
   uint32_t n_poisson_fp64;  // Poisson draws that needed an FP64 decision (call total)
 };

@@ -110,7 +110,8 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
     parts = synth.Particles(rng.integers(0, 3, n).astype(np.int32), rng.uniform(1e3, 1e5, n).astype(np.float32),
                             rng.uniform(-5.2, 5.2, n).astype(np.float32), rng.uniform(-3.2, 3.2, n).astype(np.float32),
                             off)
-    ref = O.simulate(ogeo, O.OracleParams(prm), parts, seed=4).cells64
+    oracle = O.simulate(ogeo, O.OracleParams(prm), parts, seed=4)
+    ref, canon = oracle.cells64, oracle.cells_canon
     s = fcs.Simulator(geo, prm)
     try:
         d = s.to_device(parts)
@@ -145,6 +146,12 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             fcs.fcs_simulate_events_host(s.geo, s.prm, s.ws, *(a.numpy() for a in pin), 4, 0, fcs.make_config(),
                                          *(host[k].numpy() for k in ("cell_ids", "cell_E", "event_offsets")))
             check(host)
+        det = fcs.MODE_DETERMINISTIC  # the canonical fold, bit for bit
+        for r in (s.simulate(d, 4, mode=det), s.simulate(d, 4, mode=det, wave_events=40),
+                  s.simulate(d, 4, mode=det, block=256), s.simulate(d, 4, mode=det)):
+            check(r)
+            ev, cell = np.nonzero(ref)
+            assert np.array_equal(r["cell_E"][:nnz].cpu().numpy().view(np.uint32), canon[ev, cell].view(np.uint32))
         check(s.simulate(d, 4, block=256))  # the rows were left zero
     finally:
         s.close()
