@@ -155,3 +155,19 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
         check(s.simulate(d, 4, block=256))  # the rows were left zero
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("n, E", [(1, 1.0e6), (3, 3.0e5), (340, 3.0e3), (380, 3.0e3), (1500, 1.0e4)])
+def test_long_segments(geo, prm, ogeo, n, E):
+    """Cells of many records in deterministic mode: few tasks with thousands of
+    records, about as many tasks as the fold's table takes, and more than that
+    with fewer and with more than 1024 records."""
+    parts = synth.Particles(np.zeros(n, np.int32), np.full(n, E, np.float32), np.full(n, 0.22, np.float32),
+                            np.zeros(n, np.float32), np.array([0, n], np.int64))
+    canon = O.simulate(ogeo, O.OracleParams(prm), parts, seed=6).cells_canon
+    s = fcs.Simulator(geo, prm)
+    try:
+        got = s.simulate(s.to_device(parts), 6, mode=fcs.MODE_DETERMINISTIC, dense=True)["cells"].cpu().numpy()
+        assert np.array_equal(got.view(np.uint32), canon.view(np.uint32))
+    finally:
+        s.close()
