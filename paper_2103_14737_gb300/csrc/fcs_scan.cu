@@ -4,12 +4,12 @@
 // The element count may live in device memory, so the launch needs no host
 // synchronisation.
 //
-// Persistent CTAs take tiles of 256 threads x 4, 16 or 32 elements in
+// Persistent CTAs take tiles of 256 threads x 4 or 16 elements in
 // increasing order from an atomic ticket: small tiles where 4096-element ones
-// would leave most SMs without one, large ones for the hit offsets of long
-// task lists.  A tile publishes its aggregate, then (after looking back
-// over its predecessors) its inclusive prefix, each as one 64-bit status word
-// [flag:2 | value:62].  A tile waits only on tiles with smaller tickets, which
+// would leave most SMs without one (the hit offsets of long task lists have a
+// kernel of their own, k_scan_hits).  A tile publishes its aggregate, then
+// (after looking back over its predecessors) its inclusive prefix, each as one
+// 64-bit status word [flag:2 | value:62].  A tile waits only on tiles with smaller tickets, which
 // CTAs that are already running hold, so the waits end; each wait is bounded
 // all the same and sets FCS_FLAG_WAIT_TIMEOUT when it gives up.  Input and
 // output move through shared memory (coalesced), each thread scanning
@@ -23,8 +23,6 @@
 // Where a small tile's tasks are long (more granules than tasks), a thread
 // takes a granule and searches the tile's offsets for its task; else each task
 // writes its own granules.
-#include <atomic>
-
 #include "fcs_internal.cuh"
 #include "fcs_lookback.cuh"
 
@@ -34,7 +32,7 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;  // elements per thread
 constexpr int kScanTile = kScanThreads * kScanItems;
-constexpr int kLargeItems = 32, kSmallItems = 4;
+constexpr int kSmallItems = 4;
 constexpr int64_t kSmallScan = 1 << 21;  // scans of up to this many elements may take small tiles
 constexpr int64_t kSmallTile = kScanThreads * kSmallItems;
 
@@ -204,6 +202,165 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(const In* in, Out* out, c
   }
 }
 
+// The hit offsets and the tile map of long task lists: a warp takes 1024
+// consecutive tasks, 128 to a row, four to a lane by one 16-byte load, all
+// eight rows in flight; places come from warp scans of the lanes' sums (in 32
+// bits where the warp's counts allow), so that the tile goes through no shared
+// memory.  The general scan in tiles of 8192 spent 89 instructions a task on the
+// passes through its 64-bit tile: 86 million tasks 348 us, 225 here (four CTAs
+// an SM 238; tiles of 4096 or 16384 tasks 260 to 290), 5.5 million 33 and 28.
+constexpr int kHitRows = 8;
+constexpr int kHitWarpTasks = 128 * kHitRows;
+constexpr int kHitTile = (kScanThreads / 32) * kHitWarpTasks;
+
+// Exclusive warp sum of one T per lane; the total is added to *run.
+template <typename T>
+__device__ __forceinline__ T row_excl(T own, T* run) {
+  const int lane = threadIdx.x & 31;
+  T x = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  const T before = *run + x - own;
+  *run += __shfl_sync(0xffffffffu, x, 31);
+  return before;
+}
+
+// A lane's four tasks of a row from task i on (counts past n are 0).
+__device__ __forceinline__ int4 load_counts(const int32_t* __restrict__ in, int64_t i, int64_t n) {
+  if (i + 4 <= n) return *reinterpret_cast<const int4*>(in + i);
+  return make_int4(i < n ? in[i] : 0, i + 1 < n ? in[i + 1] : 0, i + 2 < n ? in[i + 2] : 0, 0);
+}
+
+// Their offsets, the first task's hits from b0 on, and their granules of the map.
+__device__ __forceinline__ void write_offsets(int4 v, int64_t b0, int64_t i, int64_t n, int64_t* __restrict__ out,
+                                              int32_t* __restrict__ gmap, int64_t gmap_cap) {
+  const int c[4] = {v.x, v.y, v.z, v.w};
+  int64_t b[4];
+  b[0] = b0;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) b[k] = b[k - 1] + c[k - 1];
+  if (i + 4 <= n) {
+    *reinterpret_cast<longlong2*>(out + i) = make_longlong2(b[0], b[1]);
+    *reinterpret_cast<longlong2*>(out + i + 2) = make_longlong2(b[2], b[3]);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (i + k < n) out[i + k] = b[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    // (from b to the next granule's first hit; few tasks hold one)
+    if (((0u - (uint32_t)b[k]) & (kGranule - 1)) < (uint32_t)c[k]) {
+      const int64_t e = b[k] + c[k];
+      for (int64_t g = (b[k] + kGranule - 1) / kGranule; g * kGranule < e && g < gmap_cap; ++g) gmap[g] = (int32_t)(i + k);
+    }
+  }
+}
+
+// The same for a warp whose counts may not add up in 32 bits: its total, and
+// (write) its offsets.
+__device__ __noinline__ int64_t wide_counts(const int32_t* __restrict__ in, int64_t i0, int64_t n, bool write, int64_t b0,
+                                            int64_t* __restrict__ out, int32_t* __restrict__ gmap, int64_t gmap_cap) {
+  int64_t run = 0;
+#pragma unroll 1
+  for (int r = 0; r < kHitRows; ++r) {
+    const int64_t i = i0 + 128 * r + 4 * (threadIdx.x & 31);
+    const int4 v = load_counts(in, i, n);
+    const int64_t before = row_excl<int64_t>((int64_t)v.x + v.y + v.z + v.w, &run);
+    if (write) write_offsets(v, b0 + before, i, n, out, gmap, gmap_cap);
+  }
+  return run;
+}
+
+__global__ void __launch_bounds__(kScanThreads, 3) k_scan_hits(const int32_t* __restrict__ in,
+                                                                          int64_t* __restrict__ out,
+                                                                          const int64_t* __restrict__ n_dev,
+                                                                          int64_t* total_dst, uint64_t* state,
+                                                                          int64_t cap_tiles, uint32_t* flags,
+                                                                          int32_t* __restrict__ gmap, int64_t gmap_cap) {
+  dependent_start();
+  __shared__ int64_t s_w[kScanThreads / 32];
+  __shared__ int64_t s_excl;
+  __shared__ unsigned long long s_ticket;
+  __shared__ int s_last;
+  unsigned long long* ticket = reinterpret_cast<unsigned long long*>(state);
+  unsigned long long* done = ticket + 1;
+  uint64_t* status = state + 2;
+  const int64_t n = *n_dev;
+  int64_t n_tiles = (n + kHitTile - 1) / kHitTile;
+  if (n_tiles > cap_tiles) {  // the workspace sizes the state for its arrays: never
+    if (threadIdx.x == 0) atomicOr(flags, (uint32_t)FCS_FLAG_WAIT_TIMEOUT);
+    n_tiles = 0;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  while (true) {
+    if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1ull);
+    __syncthreads();
+    const int64_t t = (int64_t)s_ticket;
+    if (t >= n_tiles) break;
+    const int64_t i0 = t * kHitTile + warp * kHitWarpTasks;
+    int4 v[kHitRows];
+    uint32_t all = 0;
+#pragma unroll
+    for (int r = 0; r < kHitRows; ++r) v[r] = load_counts(in, i0 + 128 * r + 4 * lane, n);
+#pragma unroll
+    for (int r = 0; r < kHitRows; ++r) all |= (uint32_t)(v[r].x | v[r].y | v[r].z | v[r].w);
+    // 1024 counts below 2^21 add up below 2^31
+    const bool small = !__any_sync(0xffffffffu, (all >> 21) != 0u);
+    uint32_t pre[kHitRows], run = 0;
+#pragma unroll
+    for (int r = 0; r < kHitRows; ++r) pre[r] = row_excl<uint32_t>((uint32_t)(v[r].x + v[r].y + v[r].z + v[r].w), &run);
+    const int64_t warp_total = small ? (int64_t)run : wide_counts(in, i0, n, false, 0, out, gmap, gmap_cap);
+    if (lane == 0) s_w[warp] = warp_total;
+    __syncthreads();
+    if (warp == 0) {
+      int64_t total = 0;
+#pragma unroll
+      for (int w = 0; w < kScanThreads / 32; ++w) total += s_w[w];
+      int64_t excl = 0;
+      if (t) {
+        if (lane == 0) atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagAgg | (uint64_t)total);
+        excl = look_back(status, t, flags);
+      }
+      if (lane == 0) {
+        atomicExch(reinterpret_cast<unsigned long long*>(status + t), kFlagPrefix | (uint64_t)(excl + total));
+        s_excl = excl;
+        if (t == n_tiles - 1) *total_dst = excl + total;
+      }
+    }
+    __syncthreads();
+    int64_t b0 = s_excl;
+    for (int w = 0; w < warp; ++w) b0 += s_w[w];
+    if (small) {
+#pragma unroll
+      for (int r = 0; r < kHitRows; ++r)
+        write_offsets(v[r], b0 + (int64_t)pre[r], i0 + 128 * r + 4 * lane, n, out, gmap, gmap_cap);
+    } else {
+      wide_counts(in, i0, n, true, b0, out, gmap, gmap_cap);
+    }
+    __syncthreads();  // s_w and s_ticket are reused
+  }
+  // every CTA has left its loop (and its look-backs) before it counts itself
+  // done; the last one resets the state
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = atomicAdd(done, 1ull) == (unsigned long long)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_last) {
+    __threadfence();
+    for (int64_t i = threadIdx.x; i < n_tiles; i += kScanThreads) status[i] = 0;
+    if (threadIdx.x == 0) {
+      if (n_tiles == 0) *total_dst = 0;
+      *ticket = 0;
+      *done = 0;
+    }
+  }
+}
+
 }  // namespace
 
 int64_t scan_state_words(int64_t max_elements, bool small_tiles) {
@@ -226,18 +383,7 @@ static cudaError_t launch_scan(const In* in, Out* out, const int64_t* n_dev, int
                                int64_t* total_dst, int64_t base_from_dst, ScanTmp tmp, cudaStream_t s,
                                int32_t* gmap = nullptr, int64_t gmap_cap = 0) {
   constexpr size_t smem = scan_smem_bytes(ITEMS);
-  if constexpr (smem > 48 * 1024) {  // above the default limit: opt in, once per device
-    constexpr int kMaxDevices = 64;
-    static std::atomic<bool> opted[kMaxDevices];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = -1;
-    if (dev < 0 || !opted[dev].load(std::memory_order_acquire)) {
-      const cudaError_t e = cudaFuncSetAttribute(k_scan<In, GMAP, ITEMS, Out, ZERO_IN>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0) opted[dev].store(true, std::memory_order_release);
-    }
-  }
+  static_assert(smem <= 48 * 1024, "no opt-in");
   // (the status words: scan_state_words)
   return launch_dependent(k_scan<In, GMAP, ITEMS, Out, ZERO_IN>, tmp.grid, kScanThreads, smem, s, in, out, n_dev, n_host,
                           total_dst, base_from_dst ? 1 : 0, tmp.state, tmp.cap_tiles, tmp.flags, gmap, gmap_cap, -1);
@@ -292,7 +438,9 @@ cudaError_t launch_scan_hits(const int32_t* tn, int64_t* th, const int64_t* n_ta
   // 2932 tasks of 740 hits, 421,000 of 17: 28 and 16 us in tiles of 8192, 18 and 10.5 in tiles of 1024
   if (small_tiles(n_max, tmp))
     return launch_scan<int32_t, true, kSmallItems>(tn, th, n_tasks, 0, n_hits, 0, tmp, s, gmap, gmap_cap);
-  return launch_scan<int32_t, true, kLargeItems>(tn, th, n_tasks, 0, n_hits, 0, tmp, s, gmap, gmap_cap);
+  // (tn and th start on multiples of 16 bytes)
+  return launch_dependent(k_scan_hits, tmp.grid, kScanThreads, 0, s, tn, th, n_tasks, n_hits, tmp.state,
+                          tmp.cap_tiles, tmp.flags, gmap, gmap_cap);
 }
 
 }  // namespace fcs

@@ -171,3 +171,24 @@ def test_long_segments(geo, prm, ogeo, n, E):
         assert np.array_equal(got.view(np.uint32), canon.view(np.uint32))
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("n, E_first", [(90_000, 500.0), (90_001, 1.5e8), (91_351, 500.0)])
+def test_long_task_lists(geo, prm, ogeo, n, E_first):
+    """The hit offsets of more than 2^21 possible tasks: remainders of the lanes'
+    four tasks and of the warps', and a task of more than 2^21 hits, whose warp
+    adds in 64 bits."""
+    rng = np.random.default_rng(n)
+    E = rng.uniform(50.0, 500.0, n).astype(np.float32)
+    E[n // 3] = E_first
+    parts = synth.Particles(rng.integers(0, 3, n).astype(np.int32), E, rng.uniform(-4.0, 4.0, n).astype(np.float32),
+                            rng.uniform(-3.1, 3.1, n).astype(np.float32), np.array([0, n // 2, n], np.int64))
+    parts.eta[n // 3], parts.type[n // 3] = 0.2, 0
+    ref = O.simulate(ogeo, O.OracleParams(prm), parts, seed=3)
+    s = fcs.Simulator(geo, prm)
+    try:
+        got = s.simulate(s.to_device(parts), 3, mode=fcs.MODE_DETERMINISTIC, dense=True)
+        assert got["stats"]["n_hits"] == ref.n_hits and got["stats"]["n_tasks"] == ref.n_tasks
+        assert np.array_equal(got["cells"].cpu().numpy().view(np.uint32), ref.cells_canon.view(np.uint32))
+    finally:
+        s.close()
