@@ -45,28 +45,27 @@ SEED = 1
 # per clock x 152 SMs x 2070 MHz.  The lane counts are those the unit
 # microbenchmarks show (fcs_microbench; bench.py reports them as measured).
 OPS_PER_HIT = {
-    # Philox4x32-10: 10 rounds x 2 (32 x 32 -> 64-bit) multiplies
-    "mulwide": 20,
-    # Philox 20 3-input XORs; bin 6; uniforms 4; region search 6; grid index 10;
-    # deposit 4; task lookup 4
-    "int": 54,
-    # uniforms 2; (r, alpha) 2; sincos range 1; (eta, phi) 4; bounds 8;
-    # scaled indices 4; certification compares 8
-    "fp32": 29,
+    # Philox4x32-10 (32 x 32 -> 64-bit) multiplies: 8 rounds x 2 and one in each
+    # of the first two, whose other factors are the task's
+    "mulwide": 18,
+    # Philox 19 3-input XORs; bin 9; uniforms 2; phi wrap and cell index 8;
+    # deposit 6; task lookup 6
+    "int": 50,
+    # (r, alpha) 2; sincos range 1; r cos, r sin 2; (eta, phi) index maps 2 and
+    # clamps 2; rounding 2; certification 4, bounds 2, compares 2; deposit 1
+    "fp32": 20,
     # sin, cos
     "mufu": 2,
-    # 32-bit shared-memory words read from the staged tables: the hit's region
-    # (eta_lo, 1/deta, phi_lo, 1/dphi, n_eta, n_phi, cell offset), its r bin
-    # (lo, width, hi) and alpha bin (lo, width); the per-task parameters are
-    # per task, not per hit
-    "lds": 12,
+    # 32-bit shared-memory words: the hit's r bin (lo, width) and alpha bin (lo,
+    # width); the staged task's values are per task, not per hit
+    "lds": 4,
 }
 SMS, SM_MAX_MHZ = 152, 2070.0
 # DRAM bytes per hit of the hit kernel, from the committed ncu summary of its
-# 16-event capture (94.18 MB read + 4.50 MB written for 21,805,787 hits;
+# 16-event capture (94.43 MB read + 3.78 MB written for 21,805,787 hits;
 # traffic grows with the hits): valid for the kernel version captured there,
 # None after a kernel change.
-K_HITS_DRAM_BYTES_PER_HIT = 4.53
+K_HITS_DRAM_BYTES_PER_HIT = 4.50
 LANES_PER_SM_CLK = {"mulwide": 32, "int": 64, "fp32": 128, "mufu": 16, "lds": 32}
 
 

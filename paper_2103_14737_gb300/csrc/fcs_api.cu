@@ -464,14 +464,14 @@ struct CallArgs {
 // 4 TeV 64 x 4 884 and 879; from and to host buffers, in waves: 500 x 1 1687 and
 // 196, 64 x 8 358 and 195).  Deterministic calls, which also scan and fold by
 // cells, gain up to twice that: 500 x 1 942 and 153, 500 x 8 1102 and 498, 64 x 16
-// 305 and 271, 64 x 32 333 and 334.  Only the hit kernel's default shape marks.
+// 305 and 271, 64 x 32 333 and 334.
 constexpr int32_t kSparseRows = 32;
 constexpr int64_t kSparseParticles = 8, kSparseParticlesDet = 16;
 bool sparse_events(const CallArgs& a, int32_t rows) {
   const fcs_config& c = a.cfg;
   const int64_t limit = c.mode == FCS_MODE_DETERMINISTIC ? kSparseParticlesDet : kSparseParticles;
   const bool dumps = a.dbg && (a.dbg->hit_cell || a.dbg->hit_bin);
-  return c.batched == 1 && (c.block == 0 || c.block == 128) && !a.cells_out && !dumps &&
+  return c.batched == 1 && !a.cells_out && !dumps &&
          rows >= kSparseRows && a.n_particles <= limit * a.n_events &&
          a.geo->d.acc_stride >> kMarkShift <= kMaxRowMarks;
 }

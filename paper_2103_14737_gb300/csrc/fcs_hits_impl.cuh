@@ -50,7 +50,7 @@ static cudaError_t launch_hits_block(const HitKParams& kp, const Launch& L) {
   if constexpr (MODE != kModeGrad) {
     if (kp.dbg_hit_cell || kp.dbg_hit_bin) return launch_hits_kernel<BLOCK, MODE, true>(kp, L);
   }
-  if constexpr (MODE != kModeGrad && BLOCK == 128) {
+  if constexpr (MODE != kModeGrad) {
     if (kp.w.marks) return launch_hits_kernel<BLOCK, MODE, false, true>(kp, L);
   }
   return launch_hits_kernel<BLOCK, MODE, false>(kp, L);

@@ -316,8 +316,8 @@ __device__ __forceinline__ const float* event_ehit(const float* __restrict__ tas
 // and a warp that folds 32 neighbouring cells folds for the few that are not.
 // So a warp reads the offsets of 64 cells at a time, puts the cells to fold into
 // a queue of its own and folds 32 of them whenever it holds that many: 33 hard
-// scatters 52 to 26 us, 64 pile-up events 137 to 108 (256 cells at a time, 5 CTAs
-// per SM: 28 and 123).
+// scatters 52 to 26 us, the whole call of 64 pile-up events 1478 to 1431 (256
+// cells at a time, 5 CTAs per SM: 28 us and 1446).
 constexpr int kFoldWarps = 8, kFoldLoads = 2;
 constexpr int kFoldQueue = 32 * (kFoldLoads + 1);  // < 32 left after the folds + the new
 

@@ -125,10 +125,11 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             assert np.array_equal(ids, cell[:nnz])
             np.testing.assert_allclose(E, ref[ev, cell][:nnz], rtol=1e-5)
 
-        general = s.simulate(d, 4, block=256, capacity=1 << 18)  # reads every cell
+        general = s.simulate(d, 4, dense=True, capacity=1 << 18)  # reads every cell
         check(general)
         check(s.simulate(d, 4))
-        check(s.simulate(d, 4, wave_events=40))
+        check(s.simulate(d, 4, block=256))
+        check(s.simulate(d, 4, block=512, wave_events=40))
         nnz = int(general["event_offsets"][-1])
         small = s.simulate(d, 4, capacity=nnz - 3, check=False)
         assert small["status"] == fcs.FCS_E_RANGE
@@ -148,11 +149,11 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             check(host)
         det = fcs.MODE_DETERMINISTIC  # the canonical fold, bit for bit
         for r in (s.simulate(d, 4, mode=det), s.simulate(d, 4, mode=det, wave_events=40),
-                  s.simulate(d, 4, mode=det, block=256), s.simulate(d, 4, mode=det)):
+                  s.simulate(d, 4, mode=det, dense=True), s.simulate(d, 4, mode=det, block=256)):
             check(r)
             ev, cell = np.nonzero(ref)
             assert np.array_equal(r["cell_E"][:nnz].cpu().numpy().view(np.uint32), canon[ev, cell].view(np.uint32))
-        check(s.simulate(d, 4, block=256))  # the rows were left zero
+        check(s.simulate(d, 4, dense=True, capacity=1 << 18))  # the rows were left zero
     finally:
         s.close()
 
