@@ -193,3 +193,32 @@ def test_long_task_lists(geo, prm, ogeo, n, E_first):
         assert np.array_equal(got["cells"].cpu().numpy().view(np.uint32), ref.cells_canon.view(np.uint32))
     finally:
         s.close()
+
+
+def test_host_calls_with_new_arguments(geo, prm):
+    """Host-buffer calls on one workspace whose seeds, first events, event counts,
+    number of waves and density change from call to call, each against a device
+    call: the instantiated graph takes the new parameters or is made anew."""
+    batches = [synth.pileup(3, 5, mu_pu=20), synth.pileup(4, 6, mu_pu=20), synth.pileup(5, 2, mu_pu=20),
+               synth.single_particle(70), synth.single_particle(520)]
+    s, h = fcs.Simulator(geo, prm), fcs.Simulator(geo, prm)
+    try:
+        cap = 1 << 19
+        out = [torch.zeros(cap, dtype=torch.int32).pin_memory(), torch.zeros(cap).pin_memory()]
+        for k, (i, seed, first) in enumerate([(1, 9, 0), (0, 1, 0), (0, 2, 0), (0, 2, 7), (1, 2, 7), (2, 3, 0), (0, 1, 0),
+                                              (3, 1, 0), (3, 2, 0), (4, 1, 0), (4, 5, 1), (0, 1, 0)]):
+            parts = batches[i]
+            pin = [torch.as_tensor(a).pin_memory().numpy()
+                   for a in (parts.type, parts.E, parts.eta, parts.phi, parts.event_offsets)]
+            off = torch.zeros(parts.n_events + 1, dtype=torch.int64).pin_memory()
+            out[0].fill_(-1)
+            fcs.fcs_simulate_events_host(h.geo, h.prm, h.ws, *pin, seed, first, fcs.make_config(), out[0].numpy(),
+                                         out[1].numpy(), off.numpy())
+            ref = s.simulate(s.to_device(parts), seed, first_event=first, capacity=cap)
+            nnz = int(off[-1])
+            assert torch.equal(off, ref["event_offsets"].cpu()), k
+            assert torch.equal(out[0][:nnz], ref["cell_ids"][:nnz].cpu()), k
+            torch.testing.assert_close(out[1][:nnz], ref["cell_E"][:nnz].cpu(), rtol=1e-5, atol=1e-3)
+    finally:
+        s.close()
+        h.close()
