@@ -472,7 +472,7 @@ bool sparse_events(const CallArgs& a, int32_t rows) {
   const fcs_config& c = a.cfg;
   const int64_t limit = c.mode == FCS_MODE_DETERMINISTIC ? kSparseParticlesDet : kSparseParticles;
   const bool dumps = a.dbg && (a.dbg->hit_cell || a.dbg->hit_bin);
-  return c.batched == 1 && !a.cells_out && !dumps &&
+  return c.batched == 1 && !dumps &&
          rows >= kSparseRows && a.n_particles <= limit * a.n_events &&
          a.geo->d.acc_stride >> kMarkShift <= kMaxRowMarks;
 }
@@ -581,7 +581,8 @@ int enqueue_range_reduce(const CallArgs& a, WsDev w, int32_t ev_lo, int32_t rows
   if (a.cfg.mode == FCS_MODE_DETERMINISTIC)
     FCS_CUDA(launch_det_reduce(a.geo->d, w, rows, key_task_bits, ws->cell_off, a.parts.event_offsets, ev_lo, tmp, L));
   if (w.marks) {
-    FCS_CUDA(launch_compact_sparse(a.geo->d, w, rows, ev_lo, tmp, a.cell_ids, a.cell_E, a.event_offsets_out, a.capacity, L));
+    FCS_CUDA(launch_compact_sparse(a.geo->d, w, rows, ev_lo, tmp, a.cells_out, a.cell_ids, a.cell_E, a.event_offsets_out,
+                                   a.capacity, L));
     return FCS_OK;
   }
   FCS_CUDA(launch_compact(a.geo->d, w, rows, ev_lo, tmp, a.cells_out, a.cell_ids, a.cell_E, a.event_offsets_out,

@@ -224,6 +224,9 @@ constexpr int kSparseParts = 304;    // parts wanted of all rows
 //   here                          16       18        21        90        300
 // (marks of 4096 cells 133 us at 500 x 1; parts for 608 CTAs of 4 an SM, 8
 // groups in flight 25.)
+// DENSE: also the dense rows, zeros first and the marked cells over them (500
+// single electrons, the whole call: 387 us by k_compact_one, 179 here).
+template <bool DENSE>
 __global__ void __launch_bounds__(kCThreads, kSparseCtas) k_compact_sparse(const CompactArgs A, uint8_t* __restrict__ marks) {
   dependent_start();
   __shared__ uint16_t s_list[kMaxRowMarks];  // the part's marked groups, in order
@@ -253,6 +256,16 @@ __global__ void __launch_bounds__(kCThreads, kSparseCtas) k_compact_sparse(const
     if (t >= n_t) break;
     const int64_t row = t / A.cpr;
     const int mark0 = (int)(t % A.cpr) * part_marks;
+    float* const dense = DENSE ? A.cells_out + (A.ev_lo + row) * (int64_t)A.n_cells : nullptr;
+    if constexpr (DENSE) {  // (the barriers below order the zeros before the cells)
+      const int c0 = mark0 << kMarkShift, c1 = min((mark0 + part_marks) << kMarkShift, A.n_cells);
+      if ((A.n_cells & 3) == 0 && (reinterpret_cast<uintptr_t>(dense) & 15) == 0) {
+        for (int c = c0 + 4 * tid; c < c1; c += 4 * kCThreads)
+          *reinterpret_cast<float4*>(dense + c) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      } else {
+        for (int c = c0 + tid; c < c1; c += kCThreads) dense[c] = 0.0f;
+      }
+    }
     double2* const cells = reinterpret_cast<double2*>(A.acc + row * A.stride) + lane;
     {
       const int first = mark0 + warp * seg;
@@ -331,14 +344,23 @@ __global__ void __launch_bounds__(kCThreads, kSparseCtas) k_compact_sparse(const
         if (nx || ny) cells[32 * group] = make_double2(0.0, 0.0);
         int64_t p = pos + __popc(mx & below) + __popc(my & below);
         const int c = (group << kMarkShift) + 2 * lane;
-        if (nx && p < A.capacity && A.cell_ids) {
-          A.cell_ids[p] = c;
-          A.cell_E[p] = acc_to_f32(v[j].x);
+        const bool px = p < A.capacity && A.cell_ids, py = p + (nx ? 1 : 0) < A.capacity && A.cell_ids;
+        if (nx && (DENSE || px)) {
+          const float E = acc_to_f32(v[j].x);
+          if (DENSE) dense[c] = E;
+          if (px) {
+            A.cell_ids[p] = c;
+            A.cell_E[p] = E;
+          }
         }
         p += nx ? 1 : 0;
-        if (ny && p < A.capacity && A.cell_ids) {
-          A.cell_ids[p] = c + 1;
-          A.cell_E[p] = acc_to_f32(v[j].y);
+        if (ny && (DENSE || py)) {
+          const float E = acc_to_f32(v[j].y);
+          if (DENSE) dense[c + 1] = E;
+          if (py) {
+            A.cell_ids[p] = c + 1;
+            A.cell_E[p] = E;
+          }
         }
         pos += __popc(mx) + __popc(my);
       }
@@ -384,16 +406,17 @@ cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo
   return launch_dependent(kernel, grid, kCThreads, 0, L.s, A);
 }
 
-cudaError_t launch_compact_sparse(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, int32_t* cell_ids,
-                                  float* cell_E, int64_t* event_offsets_out, int64_t capacity, const Launch& L) {
+cudaError_t launch_compact_sparse(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, float* cells_out,
+                                  int32_t* cell_ids, float* cell_E, int64_t* event_offsets_out, int64_t capacity,
+                                  const Launch& L) {
   if (rows <= 0) return cudaSuccess;
   // (no more parts than the row has chunks: the scan state's size)
   const int parts = std::max(1, std::min((g.n_cells + kChunk - 1) / kChunk, kSparseParts / rows));
   const int64_t n_parts = (int64_t)rows * parts;
   const int grid = (int)std::min<int64_t>(n_parts, (int64_t)L.num_sms * kSparseCtas);
   const CompactArgs A{w.acc, g.n_cells, g.acc_stride, parts, ev_lo, 0, n_parts, tmp.state, tmp.cap_tiles, tmp.flags,
-                      &w.sizes->nnz_total, nullptr, cell_ids, cell_E, event_offsets_out, capacity};
-  return launch_dependent(k_compact_sparse, grid, kCThreads, 0, L.s, A, w.marks);
+                      &w.sizes->nnz_total, cells_out, cell_ids, cell_E, event_offsets_out, capacity};
+  return launch_dependent(cells_out ? k_compact_sparse<true> : k_compact_sparse<false>, grid, kCThreads, 0, L.s, A, w.marks);
 }
 
 int64_t compact_chunks(int32_t n_cells, int32_t rows) {

@@ -402,10 +402,11 @@ cudaError_t launch_compact(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo
                            int32_t* cell_ids, float* cell_E, int64_t* event_offsets_out, int64_t capacity,
                            int max_ctas, const Launch& L);
 
-// The same for rows whose deposits w.marks tells (no dense output): reads and
+// The same for rows whose deposits w.marks tells: reads and
 // zeroes the marked cells only, and the marks.
-cudaError_t launch_compact_sparse(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, int32_t* cell_ids,
-                                  float* cell_E, int64_t* event_offsets_out, int64_t capacity, const Launch& L);
+cudaError_t launch_compact_sparse(const GeoDev& g, WsDev w, int32_t rows, int32_t ev_lo, ScanTmp tmp, float* cells_out,
+                                  int32_t* cell_ids, float* cell_E, int64_t* event_offsets_out, int64_t capacity,
+                                  const Launch& L);
 int64_t compact_chunks(int32_t n_cells, int32_t rows);
 
 // fcs_sort.cu

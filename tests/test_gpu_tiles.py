@@ -125,7 +125,7 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             assert np.array_equal(ids, cell[:nnz])
             np.testing.assert_allclose(E, ref[ev, cell][:nnz], rtol=1e-5)
 
-        general = s.simulate(d, 4, dense=True, capacity=1 << 18)  # reads every cell
+        general = s.simulate(d, 4, debug_hits=1, capacity=1 << 18)  # reads every cell
         check(general)
         check(s.simulate(d, 4))
         check(s.simulate(d, 4, block=256))
@@ -149,11 +149,20 @@ def test_sparse_events(geo, prm, ogeo, n_events, share):
             check(host)
         det = fcs.MODE_DETERMINISTIC  # the canonical fold, bit for bit
         for r in (s.simulate(d, 4, mode=det), s.simulate(d, 4, mode=det, wave_events=40),
-                  s.simulate(d, 4, mode=det, dense=True), s.simulate(d, 4, mode=det, block=256)):
+                  s.simulate(d, 4, mode=det, debug_hits=1), s.simulate(d, 4, mode=det, block=256)):
             check(r)
             ev, cell = np.nonzero(ref)
             assert np.array_equal(r["cell_E"][:nnz].cpu().numpy().view(np.uint32), canon[ev, cell].view(np.uint32))
-        check(s.simulate(d, 4, dense=True, capacity=1 << 18))  # the rows were left zero
+        for mode in (fcs.MODE_ATOMIC, det):  # the dense rows too, all of them written
+            dense = dict(out, cells=torch.full((n_events, s.n_cells), -1.0, device="cuda"))
+            check(s.simulate(d, 4, mode=mode, outputs=dense))
+            want = torch.zeros_like(dense["cells"])
+            ev, cell = (torch.as_tensor(a, device="cuda") for a in np.nonzero(ref))
+            want[ev, cell] = dense["cell_E"][:nnz]
+            assert torch.equal(dense["cells"], want)
+            only = s.simulate(d, 4, mode=mode, outputs=dict(cells=torch.full_like(want, -1.0)), wave_events=40)["cells"]
+            torch.testing.assert_close(only, want, rtol=1e-5, atol=1e-3)
+        check(s.simulate(d, 4, debug_hits=1, capacity=1 << 18))  # the rows were left zero
     finally:
         s.close()
 
